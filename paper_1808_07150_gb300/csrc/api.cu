@@ -388,9 +388,9 @@ static int build_bwd_table(spdhg_ctx* ctx, cudaStream_t s) {
   ctx->bwd_table = 0;
   const DevGeom& g = ctx->dg;
   if (g.tune[SPDHG_TUNE_BWD_TABLE] == 1 || !backward_table_possible(g)) return SPDHG_OK;
-  const size_t cols = (size_t)((g.nx + 3) / 4) * ((g.ny + 3) / 4) * 16;
-  const size_t V = (size_t)g.V;
-  unsigned char* cnt = nullptr;
+  const size_t recs = backward_table_recs(g);
+  const size_t V = (size_t)backward_table_stages(g);
+  unsigned short* cnt = nullptr;
   unsigned *bad = nullptr, *starts = nullptr, *totals = nullptr;
   int status = SPDHG_OK;
   auto release = [&]() {
@@ -399,8 +399,8 @@ static int build_bwd_table(spdhg_ctx* ctx, cudaStream_t s) {
     ctx_free(ctx, starts);
     ctx_free(ctx, totals);
   };
-  if (ctx_malloc(ctx, (void**)&cnt, V * cols) != cudaSuccess || ctx_malloc(ctx, (void**)&bad, sizeof(unsigned)) != cudaSuccess ||
-      ctx_malloc(ctx, (void**)&starts, V * cols * sizeof(unsigned)) != cudaSuccess ||
+  if (ctx_malloc(ctx, (void**)&cnt, V * recs * sizeof(unsigned short)) != cudaSuccess || ctx_malloc(ctx, (void**)&bad, sizeof(unsigned)) != cudaSuccess ||
+      ctx_malloc(ctx, (void**)&starts, V * recs * sizeof(unsigned)) != cudaSuccess ||
       ctx_malloc(ctx, (void**)&totals, V * sizeof(unsigned)) != cudaSuccess) {
     cudaGetLastError();
     release();
@@ -426,14 +426,14 @@ static int build_bwd_table(spdhg_ctx* ctx, cudaStream_t s) {
   }
   size_t free_b = 0, total_b = 0;
   cudaMemGetInfo(&free_b, &total_b);
-  const size_t need = (size_t)total * sizeof(float4) + V * cols * sizeof(int2);
+  const size_t need = (size_t)total * sizeof(float4) + V * recs * sizeof(int2);
   if (hbad || total >= (1ull << 32) || need > free_b / 10 * 4 ||
       (ctx->mem_limit && ctx->mem_used + need > ctx->mem_limit)) {
     release();
     return SPDHG_OK;
   }
   if (ctx_malloc(ctx, (void**)&ctx->bwd_items, (size_t)total * sizeof(float4) + 16) != cudaSuccess ||
-      ctx_malloc(ctx, (void**)&ctx->bwd_hdr, V * cols * sizeof(int2)) != cudaSuccess) {
+      ctx_malloc(ctx, (void**)&ctx->bwd_hdr, V * recs * sizeof(int2)) != cudaSuccess) {
     cudaGetLastError();
     ctx_free(ctx, ctx->bwd_items);
     ctx_free(ctx, ctx->bwd_hdr);
@@ -626,7 +626,6 @@ int spdhg_create(const spdhg_geometry* geom, spdhg_ctx** out) {
   const double loz = -0.5 * g.nz * g.vz;
   std::vector<SegDev> seg(S);
   std::vector<CompDev> comp(C);
-  std::vector<int> stage_pos(P);
   int p0 = 0;
   int fz_lo = taps - 1, fz_stride = g.nz;
   for (int k = 0; k < S; ++k) {
@@ -635,8 +634,6 @@ int spdhg_create(const spdhg_geometry* geom, spdhg_ctx** out) {
     split((g.seg_zmid0[k] - loz) / g.vz, seg[k].f_hi, seg[k].f_lo);
     seg[k].c0 = -1;
     seg[k].nc = 0;
-    // the backprojector's staged slot of each plane: segment k's planes follow 2k + 1 frames
-    for (int q = 0; q < g.seg_n[k]; ++q) stage_pos[p0 + q] = p0 + q + (2 * k + 1) * (taps - 1);
     p0 += g.seg_n[k];
   }
   for (int c = 0; c < C; ++c) {
@@ -661,6 +658,19 @@ int spdhg_create(const spdhg_geometry* geom, spdhg_ctx** out) {
   for (int c = 0; c < C; ++c) fz_stride = std::max(fz_stride, g.seg_n[c_seg[c]] + 3 - comp[c].jlo);
   fz_stride += fz_lo;
   fz_stride = std::max(fz_stride, fz_lo + g.nz);
+  DevGeom& d = ctx->dg;
+  d.nx = g.nx;
+  d.ny = g.ny;
+  d.nz = g.nz;
+  d.V = V;
+  d.m = g.n_subsets;
+  d.bins = g.subset_kind == SPDHG_SUBSETS_BINS ? 1 : 0;
+  d.n_comp = C;
+  d.taps = taps;
+  d.inv_drp = (float)(g.vx / g.d_radial);
+  std::vector<int2> bw_slots;
+  std::vector<BwdBatch> bw_batch;
+  backward_layout(d, seg.data(), comp.data(), bw_slots, bw_batch);
   std::vector<int2> runs;
   for (int k = 0; k < S; ++k)
     for (int q0 = 0; q0 < g.seg_n[k]; q0 += 32) runs.push_back(make_int2(k, q0));
@@ -675,40 +685,32 @@ int spdhg_create(const spdhg_geometry* geom, spdhg_ctx** out) {
   if ((e = ctx_malloc(ctx, (void**)&ctx->d_comp, sizeof(CompDev) * C)) != cudaSuccess) return cleanup_fail(e);
   if ((e = cudaMemcpy(ctx->d_comp, comp.data(), sizeof(CompDev) * C, cudaMemcpyHostToDevice)) != cudaSuccess) return cleanup_fail(e);
   if ((e = ctx_malloc(ctx, (void**)&ctx->d_seg, sizeof(SegDev) * S)) != cudaSuccess) return cleanup_fail(e);
-  if ((e = ctx_malloc(ctx, (void**)&ctx->d_stage_pos, sizeof(int) * P)) != cudaSuccess) return cleanup_fail(e);
+  if ((e = ctx_malloc(ctx, (void**)&ctx->d_bw_slots, sizeof(int2) * bw_slots.size())) != cudaSuccess) return cleanup_fail(e);
+  if ((e = ctx_malloc(ctx, (void**)&ctx->d_bw_batch, sizeof(BwdBatch) * bw_batch.size())) != cudaSuccess) return cleanup_fail(e);
+  if ((e = cudaMemcpy(ctx->d_bw_batch, bw_batch.data(), sizeof(BwdBatch) * bw_batch.size(), cudaMemcpyHostToDevice)) != cudaSuccess) return cleanup_fail(e);
   if ((e = cudaMemcpy(ctx->d_view, view.data(), sizeof(float4) * V, cudaMemcpyHostToDevice)) != cudaSuccess) return cleanup_fail(e);
   if ((e = cudaMemcpy(ctx->d_rad, rad.data(), sizeof(float4) * R, cudaMemcpyHostToDevice)) != cudaSuccess) return cleanup_fail(e);
   if ((e = cudaMemcpy(ctx->d_rs, rs.data(), sizeof(float4) * R * C, cudaMemcpyHostToDevice)) != cudaSuccess) return cleanup_fail(e);
   if ((e = cudaMemcpy(ctx->d_seg, seg.data(), sizeof(SegDev) * S, cudaMemcpyHostToDevice)) != cudaSuccess) return cleanup_fail(e);
-  if ((e = cudaMemcpy(ctx->d_stage_pos, stage_pos.data(), sizeof(int) * P, cudaMemcpyHostToDevice)) != cudaSuccess) return cleanup_fail(e);
+  if ((e = cudaMemcpy(ctx->d_bw_slots, bw_slots.data(), sizeof(int2) * bw_slots.size(), cudaMemcpyHostToDevice)) != cudaSuccess) return cleanup_fail(e);
   if ((e = ctx_malloc(ctx, (void**)&ctx->d_runs, sizeof(int2) * runs.size())) != cudaSuccess) return cleanup_fail(e);
   if ((e = ctx_malloc(ctx, (void**)&ctx->d_view_inv, sizeof(float2) * V)) != cudaSuccess) return cleanup_fail(e);
   if ((e = cudaMemcpy(ctx->d_view_inv, view_inv.data(), sizeof(float2) * V, cudaMemcpyHostToDevice)) != cudaSuccess) return cleanup_fail(e);
   if ((e = cudaMemcpy(ctx->d_runs, runs.data(), sizeof(int2) * runs.size(), cudaMemcpyHostToDevice)) != cudaSuccess) return cleanup_fail(e);
 
-  DevGeom& d = ctx->dg;
-  d.nx = g.nx;
-  d.ny = g.ny;
-  d.nz = g.nz;
   d.R = R;
-  d.V = V;
   d.P = P;
-  d.m = g.n_subsets;
-  d.bins = g.subset_kind == SPDHG_SUBSETS_BINS ? 1 : 0;
   d.n_seg = S;
-  d.n_comp = C;
   d.mashed = mashed ? 1 : 0;
   d.comp = ctx->d_comp;
-  d.taps = taps;
-  d.nr_max = nr_max;
   d.half_R = (float)(0.5 * (R - 1));
-  d.inv_drp = (float)(g.vx / g.d_radial);
   d.view = ctx->d_view;
   d.view_inv = ctx->d_view_inv;
   d.rad = ctx->d_rad;
   d.rs = ctx->d_rs;
   d.seg = ctx->d_seg;
-  d.stage_pos = ctx->d_stage_pos;
+  d.bw_slots = ctx->d_bw_slots;
+  d.bw_batch = ctx->d_bw_batch;
   d.n_runs = (int)runs.size();
   d.runs = ctx->d_runs;
   for (int w = 0; w <= 16; ++w) {
@@ -730,7 +732,7 @@ int spdhg_create(const spdhg_geometry* geom, spdhg_ctx** out) {
 
 void spdhg_destroy(spdhg_ctx* ctx) {
   if (!ctx) return;
-  void* ptrs[] = {ctx->d_view, ctx->d_view_inv, ctx->d_rad, ctx->d_rs, ctx->d_runs, ctx->d_seg, ctx->d_comp, ctx->d_stage_pos, ctx->b, ctx->r, ctx->mult, ctx->side,
+  void* ptrs[] = {ctx->d_view, ctx->d_view_inv, ctx->d_rad, ctx->d_rs, ctx->d_runs, ctx->d_seg, ctx->d_comp, ctx->d_bw_slots, ctx->d_bw_batch, ctx->b, ctx->r, ctx->mult, ctx->side,
                   ctx->x[0], ctx->x[1], ctx->z, ctx->T, ctx->y, ctx->sigma, ctx->wdy, ctx->q[0], ctx->q[1],
                   ctx->w[0], ctx->w[1], ctx->zw, ctx->q2[0], ctx->q2[1], ctx->tgv_b, ctx->tmp_sino, ctx->tmp_img, ctx->tmp_img2, ctx->em_sens, ctx->bwd_items, ctx->bwd_hdr, ctx->fwd_part, ctx->fwd_tickets,
                   ctx->red, ctx->red_out};
@@ -829,6 +831,10 @@ int spdhg_backproject(spdhg_ctx* ctx, const float* y, float* x, int subset, void
   BwdArgs a{};
   a.w = w;
   a.out = x;
+  if (subset >= 0 && ctx->bwd_table == 1) {
+    a.items = ctx->bwd_items;
+    a.hdr = ctx->bwd_hdr;
+  }
   CK(launch_backward(ctx->dg, subset, BWD_OUT, a, s));
   return SPDHG_OK;
 }
@@ -1341,6 +1347,8 @@ int spdhg_osem(spdhg_ctx* ctx, const spdhg_params* params, int mlem, float* x_in
       CK(launch_backward(ctx->dg, sub, BWD_OUT, a, s));
     }
     ctx->em_sens_kind = kind;
+    if (!mlem)
+      if (int st = build_bwd_table(ctx, s)) return st;
   }
   // the iterate: u0 from the caller, or ones (Eq. EQU:MLEM needs a positive start)
   float* u = ctx->x[0];
@@ -1382,6 +1390,10 @@ int spdhg_osem(spdhg_ctx* ctx, const spdhg_params* params, int mlem, float* x_in
         ba.w = ratio;
         ba.x = u;
         ba.T = ctx->em_sens + (size_t)(mlem ? 0 : k) * N;
+        if (!mlem && ctx->bwd_table == 1) {
+          ba.items = ctx->bwd_items;
+          ba.hdr = ctx->bwd_hdr;
+        }
         e = launch_backward(ctx->dg, sub, BWD_EM, ba, s);
       }
       if (e != cudaSuccess) status = fail(ctx, SPDHG_ERR_CUDA, std::string("EM iteration: ") + cudaGetErrorString(e));

@@ -1,0 +1,161 @@
+// Backprojector: launch layout per geometry, tap-item table, dispatch over the tap counts.
+#include <math.h>
+
+#include <algorithm>
+#include <vector>
+
+#include "backward.cuh"
+
+namespace spdhg {
+
+// Tile, staged rows and component batches of a geometry (host; fills the bw_* fields of g and
+// slot / len of comp).  slots receives per batch the copies (slot, plane), then the zero slots.
+void backward_layout(DevGeom& g, const SegDev* seg, CompDev* comp, std::vector<int2>& slots, std::vector<BwdBatch>& batches) {
+  const double inv = g.inv_drp;
+  const int pad = g.taps - 1;
+  auto rows = [&](int cpw) {
+    // a tile of 2 cpw x 4 pixels projects onto 2 cpw |c| + 4 |s| pixels of s, at most the tile's
+    // diagonal; the kernel widens the row range by twice its bin margin on both sides
+    const double diag = sqrt(4.0 * cpw * cpw + 16.0);
+    return (int)floor(diag * inv * (1.0 + 1e-5) + 4.0 * kBinMargin) + 1;
+  };
+  auto run = [&](int c) { return comp[c].qhi - comp[c].qlo + pad; };  // its planes and one frame
+  int widest = 0;
+  for (int c = 0; c < g.n_comp; ++c) widest = std::max(widest, run(c) + pad);
+  // four columns per warp share a block's set-up and a warp's item records (171 x 171: 98 us against
+  // 149 with one column, 128 x 128: 35 against 40); one column per warp where four would leave fewer
+  // than two blocks per SM, or rows too long for shared memory
+  const long long tiles4 = (long long)((g.nx + 7) / 8) * ((g.ny + 3) / 4);
+  g.bw_cpw = tiles4 >= 2 * 152 && (size_t)rows(4) * widest * sizeof(float) <= 80 * 1024 ? 4 : 1;
+  g.bw_rows = rows(g.bw_cpw);
+  g.bw_cand = (int)floor(1.41422 * inv + 2.0 * kBinMargin) + 1;
+  // batches of components whose staged rows fit the buffer: 36 KB leave room for four blocks per SM
+  // (171 x 171 x 92, three segments: 36 KB 97.7 us, 44 KB 108.7, 24 KB 115)
+  const int room = 36 * 1024 / (int)sizeof(float) / g.bw_rows;
+  batches.clear();
+  slots.clear();
+  g.bw_buf = 0;
+  for (int c = 0; c < g.n_comp;) {
+    BwdBatch b{c, c, (int)slots.size(), 0, 0, pad};
+    std::vector<int2> zeros;
+    for (int k = 0; k < pad; ++k) zeros.push_back(make_int2(k, -1));
+    while (c < g.n_comp && (c == b.c0 || b.slots + run(c) <= room)) {
+      comp[c].slot = b.slots - pad;
+      comp[c].len = comp[c].qhi - comp[c].qlo + pad;
+      for (int q = comp[c].qlo; q < comp[c].qhi; ++q, ++b.slots) {
+        if (((q - comp[c].qlo) & comp[c].smask) == 0) slots.push_back(make_int2(b.slots, seg[comp[c].seg].p0 + q));
+        else zeros.push_back(make_int2(b.slots, -1));
+      }
+      for (int k = 0; k < pad; ++k) zeros.push_back(make_int2(b.slots++, -1));
+      ++c;
+    }
+    b.c1 = c;
+    b.copies = (int)slots.size() - b.first;
+    b.zeros = (int)zeros.size();
+    slots.insert(slots.end(), zeros.begin(), zeros.end());
+    batches.push_back(b);
+    g.bw_buf = std::max(g.bw_buf, (g.bw_rows * b.slots + 3) & ~3);
+  }
+  g.bw_nb = (int)batches.size();
+  // several views per stage where their rows are short: fewer barriers, fuller records
+  g.bw_views = 1;
+  if (g.bw_nb == 1) {
+    const int most = g.bins ? g.V : (g.V + g.m - 1) / g.m;
+    const int fit = std::max(1, std::min(16, room / batches[0].slots));
+    const int stages = (most + fit - 1) / fit;
+    g.bw_views = (most + stages - 1) / stages;
+    g.bw_buf = (g.bw_views * g.bw_rows * batches[0].slots + 3) & ~3;
+  }
+}
+
+// per stage: exclusive prefix sums of the warps' item counts, and the stage's total
+__global__ void __launch_bounds__(1024) k_bwd_table_scan(const unsigned short* cnt, size_t recs_per_view,
+                                                         unsigned* starts, unsigned* totals) {
+  __shared__ int scratch[33];
+  const size_t v = blockIdx.x;
+  const unsigned short* c = cnt + v * recs_per_view;
+  unsigned* st = starts + v * recs_per_view;
+  const size_t per = (recs_per_view + blockDim.x - 1) / blockDim.x;
+  const size_t lo = min(recs_per_view, threadIdx.x * per), hi = min(recs_per_view, lo + per);
+  int sum = 0;
+  for (size_t k = lo; k < hi; ++k) sum += c[k];
+  int total;
+  int run = block_exclusive_scan(sum, scratch, &total);
+  for (size_t k = lo; k < hi; ++k) {
+    st[k] = (unsigned)run;
+    run += c[k];
+  }
+  if (threadIdx.x == 0) totals[v] = (unsigned)total;
+}
+
+// one batch of at most 128 components, three taps (the item's packing), view subsets
+bool backward_table_possible(const DevGeom& g) {
+  return !g.bins && g.taps <= 3 && g.bw_nb == 1 && g.n_comp <= 128;
+}
+
+size_t backward_table_recs(const DevGeom& g) {
+  const dim3 t = bwd_tiles(g);
+  return (size_t)t.x * t.y * kBwdWarps;
+}
+
+int backward_table_stages(const DevGeom& g) { return g.m * bwd_groups(g, 0); }
+
+static cudaError_t table_pass(const DevGeom& g, int pass, unsigned short* cnt, unsigned* bad, const unsigned* starts,
+                              const unsigned* stage_base, float4* items, int2* hdr, cudaStream_t s) {
+  if (!backward_table_possible(g)) return cudaErrorInvalidValue;
+  switch (g.taps) {
+    case 1: return backward_items_nt<1>(g, pass, cnt, bad, starts, stage_base, items, hdr, s);
+    case 2: return backward_items_nt<2>(g, pass, cnt, bad, starts, stage_base, items, hdr, s);
+    default: return backward_items_nt<3>(g, pass, cnt, bad, starts, stage_base, items, hdr, s);
+  }
+}
+
+cudaError_t backward_table_count(const DevGeom& g, unsigned short* cnt, unsigned* bad, cudaStream_t s) {
+  return table_pass(g, 0, cnt, bad, nullptr, nullptr, nullptr, nullptr, s);
+}
+
+cudaError_t backward_table_starts(const DevGeom& g, const unsigned short* cnt, unsigned* starts,
+                                  unsigned* stage_totals, cudaStream_t s) {
+  k_bwd_table_scan<<<backward_table_stages(g), 1024, 0, s>>>(cnt, backward_table_recs(g), starts, stage_totals);
+  return cudaGetLastError();
+}
+
+cudaError_t backward_table_fill(const DevGeom& g, const unsigned* starts, const unsigned* stage_base,
+                                float4* items, int2* hdr, cudaStream_t s) {
+  return table_pass(g, 1, nullptr, nullptr, starts, stage_base, items, hdr, s);
+}
+
+cudaError_t launch_backward(const DevGeom& g, int subset, int mode, const BwdArgs& a, cudaStream_t s) {
+  if (a.items && !backward_table_possible(g)) return cudaErrorInvalidValue;
+  switch (g.taps) {
+    case 1: return launch_backward_nt<1>(g, subset, mode, a, s);
+    case 2: return launch_backward_nt<2>(g, subset, mode, a, s);
+    case 3: return launch_backward_nt<3>(g, subset, mode, a, s);
+    case 4: return launch_backward_nt<4>(g, subset, mode, a, s);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+__global__ void k_gather_subset(DevGeom g, int subset, const float* __restrict__ y,
+                                const float* __restrict__ mult, float* __restrict__ w) {
+  const int64_t per_view = (int64_t)g.R * g.P;
+  const int64_t n = (int64_t)subset_views(g, subset) * per_view;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    const int l = (int)(i / per_view);
+    const int64_t j = (int64_t)subset_view(g, subset, l) * per_view + (i - l * per_view);
+    const float v = (y ? y[j] : 1.f) * (mult ? mult[j] : 1.f);
+    w[i] = bin_in_subset(g, subset, (size_t)j) ? v : 0.f;
+  }
+}
+
+cudaError_t launch_gather_subset(const DevGeom& g, int subset, const float* y, const float* mult,
+                                 float* w_local, cudaStream_t s) {
+  const int64_t n = (int64_t)subset_views(g, subset) * g.R * g.P;
+  if (n == 0) return cudaSuccess;
+  int blocks = (int)((n + 255) / 256);
+  if (blocks > 152 * 16) blocks = 152 * 16;
+  k_gather_subset<<<blocks, 256, 0, s>>>(g, subset, y, mult, w_local);
+  return cudaGetLastError();
+}
+
+}  // namespace spdhg

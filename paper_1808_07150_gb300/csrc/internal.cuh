@@ -32,6 +32,13 @@ struct CompDev {
   int seg;
   int qlo, qhi, smask;
   int jlo, jhi;  // range of the tap offset j0 of any pixel of any LOR of the component (host bound)
+  int slot, len; // backprojector: staged slot taps - 1 below the component's first plane, its planes + taps - 1
+};
+
+// Components [c0, c1) whose planes the backprojector stages together: rows of `slots` floats; entries
+// first .. of the slot list are `copies` (slot, plane) copies, then `zeros` zero slots.
+struct BwdBatch {
+  int c0, c1, first, copies, zeros, slots;
 };
 
 // Geometry passed by value to every kernel.  Transaxial quantities are in pixel units (mm / vx);
@@ -45,7 +52,6 @@ struct DevGeom {
   int n_comp;            // LOR components (= n_seg without mashing)
   int mashed;            // 1: some bin sums several LORs or some plane lacks a component
   int taps;              // maximum slices a LOR crosses inside one pixel
-  int nr_max;            // maximum candidate radial bins per pixel and view
   float half_R;          // (R - 1) / 2
   float inv_drp;         // vx / d_radial: radial bins per pixel unit
   const float4* view;    // per view: cos_hi, cos_lo, sin_hi, sin_lo (exact zeros on the axes)
@@ -54,7 +60,12 @@ struct DevGeom {
   const float4* rs;      // per (radial bin, component): kappa_hi, kappa_lo, len_scale, 0
   const SegDev* seg;
   const CompDev* comp;
-  const int* stage_pos;  // plane -> its slot in the backprojector's staged rows (frames included)
+  // backprojector (backward_layout): voxel columns per warp, staged radial rows of a tile, candidate
+  // bins per column and view, component batches, most views per stage, floats of the staging buffer; the batches, and their
+  // copies (slot, plane) and zero slots
+  int bw_cpw, bw_rows, bw_cand, bw_nb, bw_views, bw_buf;
+  const BwdBatch* bw_batch;
+  const int2* bw_slots;
   int n_runs;            // plane runs of the forward projector: run k = planes [q0, q0 + 32) of one segment
   const int2* runs;      // (segment, q0) per run, segment-major
   int max_part_comps[17];  // forward: most components one block spans, by warps per block
@@ -98,7 +109,7 @@ __host__ __device__ inline bool bin_in_subset(const DevGeom& g, int subset, size
 struct Ctx;
 
 // ---------------------------------------------------------------------------------------
-// projector launches (projector.cu)
+// projector launches (forward.cu, backward.cu)
 // ---------------------------------------------------------------------------------------
 enum FwdMode { FWD_PROJECT = 0, FWD_SIGMA = 1, FWD_DATA = 2, FWD_EM = 3 };
 enum BwdMode { BWD_OUT = 0, BWD_SENS = 1, BWD_UPDATE = 2, BWD_EM = 3 };
@@ -134,25 +145,26 @@ struct BwdArgs {
   float* x;              // BWD_UPDATE, BWD_EM
   float* z;
   float inv_p;
-  // BWD_UPDATE: the tap items of every (view, tile, column), built once (null: computed in the
-  // kernel); see backward_table_count / _fill
+  // the tap items of every view, tile and warp, built once (null: computed in the kernel); see
+  // backward_table_count / _fill
   const float4* items;
   const int2* hdr;
 };
 
-// Tap-item table of the backprojector: for every view, 4 x 4 tile and column the (pair, segment)
-// items the kernel would compute, in its order.  Items are float4 (L0, L1, L2, packed): packed =
-// shared offset (16 bits) | (j0 + taps - 1 + 256) << 16 (9 bits) | segment << 25 (7 bits).  Header
-// per column: (first item, n1 | (n1 + n2) << 8 | n << 16) with n_k the items of k taps.
-// Pass 0 counts the items per column into `cnt` (bytes) and flags an item that does not fit the
-// packing in *bad; pass 1 fills the items and headers from the per-column starts.
-cudaError_t backward_table_count(const DevGeom& g, unsigned char* cnt, unsigned* bad, cudaStream_t s);
-cudaError_t backward_table_starts(const DevGeom& g, const unsigned char* cnt, unsigned* starts,
-                                  unsigned* view_totals, cudaStream_t s);
-cudaError_t backward_table_fill(const DevGeom& g, const unsigned* starts, const unsigned* view_base,
+// Tap-item table of the backprojector: the (pair, component) items of every stage, tile and warp in
+// the kernel's order (backward.cuh).  Count: items per warp, *bad set where one does not fit the
+// packing; starts: prefix sums per stage; fill: items and headers from the starts.
+cudaError_t backward_table_count(const DevGeom& g, unsigned short* cnt, unsigned* bad, cudaStream_t s);
+cudaError_t backward_table_starts(const DevGeom& g, const unsigned short* cnt, unsigned* starts,
+                                  unsigned* stage_totals, cudaStream_t s);
+cudaError_t backward_table_fill(const DevGeom& g, const unsigned* starts, const unsigned* stage_base,
                                 float4* items, int2* hdr, cudaStream_t s);
-// whether the geometry admits the table (unmashed, at most 3 taps, packing limits)
+// whether the geometry admits the table, its stages over all subsets and its records (warps) per stage
 bool backward_table_possible(const DevGeom& g);
+int backward_table_stages(const DevGeom& g);
+size_t backward_table_recs(const DevGeom& g);
+// tile, staged rows and component batches of a geometry (host tables; see backward.cu)
+void backward_layout(DevGeom& g, const SegDev* seg, CompDev* comp, std::vector<int2>& slots, std::vector<BwdBatch>& batches);
 
 cudaError_t launch_forward(const DevGeom& g, int subset, int mode, const FwdArgs& a, cudaStream_t s);
 cudaError_t launch_backward(const DevGeom& g, int subset, int mode, const BwdArgs& a, cudaStream_t s);
@@ -261,7 +273,8 @@ struct spdhg_ctx {
   float2* d_view_inv = nullptr;
   spdhg::SegDev* d_seg = nullptr;
   spdhg::CompDev* d_comp = nullptr;
-  int* d_stage_pos = nullptr;
+  int2* d_bw_slots = nullptr;
+  spdhg::BwdBatch* d_bw_batch = nullptr;
   // data
   float *b = nullptr, *r = nullptr, *mult = nullptr, *side = nullptr;
   bool has_data = false, has_mult = false, has_side = false;
