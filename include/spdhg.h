@@ -286,19 +286,20 @@ enum { SPDHG_TUNE_PRIOR_COLS = 0,   /* prior kernel: voxel columns per block, in
        SPDHG_TUNE_PRIOR_YCHUNK = 1, /* prior kernel: rows marched per block */
        SPDHG_TUNE_FWD_SPLIT = 2,    /* forward kernel: row parts of one LOR line (partial sums
                                        reduced in a fixed order) */
-       SPDHG_TUNE_FWD_WARPS = 3,    /* forward kernel: warps per block (1, 2, 4, 8 or 16); a warp
-                                       owns two runs of 32 planes, so a line's runs are spread
-                                       over ceil(runs / (2 * warps)) blocks */
+       SPDHG_TUNE_FWD_WARPS = 3,    /* forward kernel: plane tasks per block (1, 2, 4, 8 or 16, at
+                                       most 12 are used); a warp owns one task of up to four words
+                                       of 32 planes of one segment, so a line's tasks are spread
+                                       over ceil(tasks / value) blocks */
        SPDHG_TUNE_PRIOR_STAGES = 4, /* prior kernel: rows in its shared-memory pipeline (3 or 4) */
        SPDHG_TUNE_BWD_TABLE = 5,    /* backprojector of the iterations: 0 reads its (pixel, bin,
                                        segment) tap items from a table built by spdhg_setup when
                                        it fits in 40 % of the free device memory (about 7 GB at
                                        the mMR scale; same results bit for bit); 1 computes them in
                                        the kernel */
-       SPDHG_TUNE_FWD_GROUPS = 6,   /* forward projector: warps that share each plane run, each
+       SPDHG_TUNE_FWD_GROUPS = 6,   /* forward projector: warps that share each plane task, each
                                        taking every k-th pixel entry of the line (1 .. 8; their
                                        partial sums are added in a fixed order); 0 = enough for
-                                       four warps per block when a line has few plane runs */
+                                       four warps per block when a line has few plane tasks */
        SPDHG_TUNE_PRIOR_VZ = 7,     /* prior kernel: voxels per thread along z (1, 2 or 4;
                                        0 = 1) */
        SPDHG_TUNE_KNOBS = 8 };

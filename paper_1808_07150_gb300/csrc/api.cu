@@ -656,8 +656,9 @@ int spdhg_create(const spdhg_geometry* geom, spdhg_ctx** out) {
   }
   // plane q (read as min(q, n - 1)) reads slabs q - j0 - t: the highest is n - 1 - jlo
   for (int c = 0; c < C; ++c) fz_stride = std::max(fz_stride, g.seg_n[c_seg[c]] + 3 - comp[c].jlo);
+  fz_lo = (fz_lo + 3) & ~3;  // 16-byte copies of aligned columns
   fz_stride += fz_lo;
-  fz_stride = std::max(fz_stride, fz_lo + g.nz);
+  fz_stride = (std::max(fz_stride, fz_lo + g.nz) + 3) & ~3;
   DevGeom& d = ctx->dg;
   d.nx = g.nx;
   d.ny = g.ny;
@@ -671,9 +672,9 @@ int spdhg_create(const spdhg_geometry* geom, spdhg_ctx** out) {
   std::vector<int2> bw_slots;
   std::vector<BwdBatch> bw_batch;
   backward_layout(d, seg.data(), comp.data(), bw_slots, bw_batch);
-  std::vector<int2> runs;
-  for (int k = 0; k < S; ++k)
-    for (int q0 = 0; q0 < g.seg_n[k]; q0 += 32) runs.push_back(make_int2(k, q0));
+  std::vector<int4> tasks;
+  d.n_seg = S;
+  forward_layout(d, seg.data(), tasks);
   auto cleanup_fail = [&](cudaError_t e) {
     spdhg_destroy(ctx);
     return e == cudaErrorMemoryAllocation ? SPDHG_ERR_OOM : SPDHG_ERR_CUDA;
@@ -693,14 +694,13 @@ int spdhg_create(const spdhg_geometry* geom, spdhg_ctx** out) {
   if ((e = cudaMemcpy(ctx->d_rs, rs.data(), sizeof(float4) * R * C, cudaMemcpyHostToDevice)) != cudaSuccess) return cleanup_fail(e);
   if ((e = cudaMemcpy(ctx->d_seg, seg.data(), sizeof(SegDev) * S, cudaMemcpyHostToDevice)) != cudaSuccess) return cleanup_fail(e);
   if ((e = cudaMemcpy(ctx->d_bw_slots, bw_slots.data(), sizeof(int2) * bw_slots.size(), cudaMemcpyHostToDevice)) != cudaSuccess) return cleanup_fail(e);
-  if ((e = ctx_malloc(ctx, (void**)&ctx->d_runs, sizeof(int2) * runs.size())) != cudaSuccess) return cleanup_fail(e);
+  if ((e = ctx_malloc(ctx, (void**)&ctx->d_tasks, sizeof(int4) * tasks.size())) != cudaSuccess) return cleanup_fail(e);
   if ((e = ctx_malloc(ctx, (void**)&ctx->d_view_inv, sizeof(float2) * V)) != cudaSuccess) return cleanup_fail(e);
   if ((e = cudaMemcpy(ctx->d_view_inv, view_inv.data(), sizeof(float2) * V, cudaMemcpyHostToDevice)) != cudaSuccess) return cleanup_fail(e);
-  if ((e = cudaMemcpy(ctx->d_runs, runs.data(), sizeof(int2) * runs.size(), cudaMemcpyHostToDevice)) != cudaSuccess) return cleanup_fail(e);
+  if ((e = cudaMemcpy(ctx->d_tasks, tasks.data(), sizeof(int4) * tasks.size(), cudaMemcpyHostToDevice)) != cudaSuccess) return cleanup_fail(e);
 
   d.R = R;
   d.P = P;
-  d.n_seg = S;
   d.mashed = mashed ? 1 : 0;
   d.comp = ctx->d_comp;
   d.half_R = (float)(0.5 * (R - 1));
@@ -711,19 +711,7 @@ int spdhg_create(const spdhg_geometry* geom, spdhg_ctx** out) {
   d.seg = ctx->d_seg;
   d.bw_slots = ctx->d_bw_slots;
   d.bw_batch = ctx->d_bw_batch;
-  d.n_runs = (int)runs.size();
-  d.runs = ctx->d_runs;
-  for (int w = 0; w <= 16; ++w) {
-    // components spanned by the blocks of the forward projector with w warps (2 runs each)
-    int mx = 1;
-    const int rpp = 2 * std::max(w, 1);
-    for (size_t r0 = 0; r0 < runs.size(); r0 += rpp) {
-      const size_t r1 = std::min(runs.size(), r0 + rpp) - 1;
-      const int glo = runs[r0].x, ghi = runs[r1].x;
-      mx = std::max(mx, seg[ghi].c0 + seg[ghi].nc - seg[glo].c0);
-    }
-    d.max_part_comps[w] = mx;
-  }
+  d.tasks = ctx->d_tasks;
   d.fz_lo = fz_lo;
   d.fz_stride = fz_stride;
   *out = ctx;
@@ -732,7 +720,7 @@ int spdhg_create(const spdhg_geometry* geom, spdhg_ctx** out) {
 
 void spdhg_destroy(spdhg_ctx* ctx) {
   if (!ctx) return;
-  void* ptrs[] = {ctx->d_view, ctx->d_view_inv, ctx->d_rad, ctx->d_rs, ctx->d_runs, ctx->d_seg, ctx->d_comp, ctx->d_bw_slots, ctx->d_bw_batch, ctx->b, ctx->r, ctx->mult, ctx->side,
+  void* ptrs[] = {ctx->d_view, ctx->d_view_inv, ctx->d_rad, ctx->d_rs, ctx->d_tasks, ctx->d_seg, ctx->d_comp, ctx->d_bw_slots, ctx->d_bw_batch, ctx->b, ctx->r, ctx->mult, ctx->side,
                   ctx->x[0], ctx->x[1], ctx->z, ctx->T, ctx->y, ctx->sigma, ctx->wdy, ctx->q[0], ctx->q[1],
                   ctx->w[0], ctx->w[1], ctx->zw, ctx->q2[0], ctx->q2[1], ctx->tgv_b, ctx->tmp_sino, ctx->tmp_img, ctx->tmp_img2, ctx->em_sens, ctx->bwd_items, ctx->bwd_hdr, ctx->fwd_part, ctx->fwd_tickets,
                   ctx->red, ctx->red_out};

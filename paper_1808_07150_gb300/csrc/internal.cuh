@@ -66,9 +66,9 @@ struct DevGeom {
   int bw_cpw, bw_rows, bw_cand, bw_nb, bw_views, bw_buf;
   const BwdBatch* bw_batch;
   const int2* bw_slots;
-  int n_runs;            // plane runs of the forward projector: run k = planes [q0, q0 + 32) of one segment
-  const int2* runs;      // (segment, q0) per run, segment-major
-  int max_part_comps[17];  // forward: most components one block spans, by warps per block
+  int n_tasks;           // plane tasks of the forward projector, segment-major
+  const int4* tasks;     // (segment, first plane, words of 32 planes, 0)
+  int max_part_comps[17];  // forward: most components one block spans, by tasks per block
   int fz_lo;             // forward staging: zero slabs below each staged x column
   int fz_stride;         // forward staging: floats per staged x column (frames included)
   int tune[SPDHG_TUNE_KNOBS];  // launch-shape overrides (0: built-in heuristic)
@@ -136,6 +136,9 @@ int forward_split(const DevGeom& g, int subset);
 // plane parts per LOR line (blocks that share the rows of a line, each with its own planes)
 int forward_parts(const DevGeom& g);
 int forward_entry_groups(const DevGeom& g);
+int forward_tasks_per_part(const DevGeom& g);
+// plane tasks of a geometry (host table; see forward.cu)
+void forward_layout(DevGeom& g, const SegDev* seg, std::vector<int4>& tasks);
 
 struct BwdArgs {
   const float* w;        // subset-local sinogram (mult already applied)
@@ -269,7 +272,7 @@ struct spdhg_ctx {
   float4* d_view = nullptr;
   float4* d_rad = nullptr;
   float4* d_rs = nullptr;
-  int2* d_runs = nullptr;
+  int4* d_tasks = nullptr;
   float2* d_view_inv = nullptr;
   spdhg::SegDev* d_seg = nullptr;
   spdhg::CompDev* d_comp = nullptr;

@@ -119,13 +119,13 @@ extern "C" int spdhg_autotune(spdhg_ctx* ctx, int reps, int* chosen, void* strea
   {
     Knob k{SPDHG_TUNE_FWD_WARPS, true, {}};
     for (int w : {2, 4, 8, 16})
-      if (w == 2 || (g.n_runs + 1) / 2 > w / 2) k.values.push_back(w);
+      if (w == 2 || g.n_tasks > w / 2) k.values.push_back(w);
     knobs.push_back(k);
   }
   {
-    // entry groups only where a line's plane runs leave the block with few warps
+    // entry groups only where a line's plane tasks leave the block with few warps
     Knob k{SPDHG_TUNE_FWD_GROUPS, true, {}};
-    if (g.n_runs <= 6)
+    if (g.n_tasks <= 3)
       for (int eg : {1, 2, 4, 8}) k.values.push_back(eg);
     knobs.push_back(k);
   }
