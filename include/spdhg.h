@@ -290,7 +290,8 @@ enum { SPDHG_TUNE_PRIOR_COLS = 0,   /* prior kernel: voxel columns per block, in
                                        most 12 are used); a warp owns one task of up to four words
                                        of 32 planes of one segment, so a line's tasks are spread
                                        over ceil(tasks / value) blocks */
-       SPDHG_TUNE_PRIOR_STAGES = 4, /* prior kernel: rows in its shared-memory pipeline (3 or 4) */
+       SPDHG_TUNE_PRIOR_STAGES = 4, /* accepted (3 or 4) without effect: the prior kernel has no
+                                       shared-memory pipeline any more */
        SPDHG_TUNE_BWD_TABLE = 5,    /* backprojector of the iterations: 0 reads its (pixel, bin,
                                        segment) tap items from a table built by spdhg_setup when
                                        it fits in 40 % of the free device memory (about 7 GB at
@@ -300,8 +301,8 @@ enum { SPDHG_TUNE_PRIOR_COLS = 0,   /* prior kernel: voxel columns per block, in
                                        taking every k-th pixel entry of the line (1 .. 8; their
                                        partial sums are added in a fixed order); 0 = enough for
                                        four warps per block when a line has few plane tasks */
-       SPDHG_TUNE_PRIOR_VZ = 7,     /* prior kernel: voxels per thread along z (1, 2 or 4;
-                                       0 = 1) */
+       SPDHG_TUNE_PRIOR_VZ = 7,     /* accepted (1, 2 or 4) without effect: a thread of the prior
+                                       kernel holds one voxel */
        SPDHG_TUNE_KNOBS = 8 };
 
 /* Sets one launch-shape knob of the context (value 0: default).  Out-of-range values are rejected
@@ -341,7 +342,7 @@ int spdhg_run_batch(spdhg_ctx* const* ctx, const spdhg_params* params, float* co
 enum { SPDHG_KERNEL_FORWARD = 0,   /* subset projection fused with the KL dual prox */
        SPDHG_KERNEL_BACKWARD = 1,  /* subset backprojection fused with z and the primal step */
        SPDHG_KERNEL_PRIOR = 2,     /* TV / dTV / aTV dual step fused with z and the primal step */
-       SPDHG_KERNEL_TGV = 3,       /* TGV dual steps */
+       SPDHG_KERNEL_TGV = 3,       /* TGV blocks: dual step fused with the z, w and u steps */
        SPDHG_KERNEL_WSTEP = 4,     /* TGV primal step of w in data iterations */
        SPDHG_KERNEL_KINDS = 5 };
 

@@ -324,7 +324,6 @@ int spdhg::enqueue_block(spdhg_ctx* ctx, int i, cudaStream_t s) {
     ta.Tw = ctx->Tw;
     ta.sigma = ctx->sigma_prior[kblk];
     ta.inv_p = inv_p;
-    ta.bscr = ctx->tgv_b;
     {
       ProfScope ps(ctx, SPDHG_KERNEL_TGV, s);
       CK(launch_tgv(ctx->dg, ta, s));
@@ -722,7 +721,7 @@ void spdhg_destroy(spdhg_ctx* ctx) {
   if (!ctx) return;
   void* ptrs[] = {ctx->d_view, ctx->d_view_inv, ctx->d_rad, ctx->d_rs, ctx->d_tasks, ctx->d_seg, ctx->d_comp, ctx->d_bw_slots, ctx->d_bw_batch, ctx->b, ctx->r, ctx->mult, ctx->side,
                   ctx->x[0], ctx->x[1], ctx->z, ctx->T, ctx->y, ctx->sigma, ctx->wdy, ctx->q[0], ctx->q[1],
-                  ctx->w[0], ctx->w[1], ctx->zw, ctx->q2[0], ctx->q2[1], ctx->tgv_b, ctx->tmp_sino, ctx->tmp_img, ctx->tmp_img2, ctx->em_sens, ctx->bwd_items, ctx->bwd_hdr, ctx->fwd_part, ctx->fwd_tickets,
+                  ctx->w[0], ctx->w[1], ctx->zw, ctx->q2[0], ctx->q2[1], ctx->tmp_sino, ctx->tmp_img, ctx->tmp_img2, ctx->em_sens, ctx->bwd_items, ctx->bwd_hdr, ctx->fwd_part, ctx->fwd_tickets,
                   ctx->red, ctx->red_out};
   for (void* p : ptrs) ctx_free(ctx, p);
   for (auto& r : ctx->prof_pending) {
@@ -887,7 +886,6 @@ int spdhg_setup(spdhg_ctx* ctx, const spdhg_params* params, const float* x0, int
     CK(dalloc(ctx, &ctx->w[0], 3 * N));
     CK(dalloc(ctx, &ctx->w[1], 3 * N));
     CK(dalloc(ctx, &ctx->zw, 3 * N));
-    CK(dalloc(ctx, &ctx->tgv_b, 6 * N));
     CK(dalloc(ctx, &ctx->q2[0], 6 * N));
     CK(dalloc(ctx, &ctx->q2[1], 6 * N));
   }
@@ -1422,7 +1420,7 @@ int spdhg_tune(spdhg_ctx* ctx, int knob, int value) {
   if (!ctx || knob < 0 || knob >= SPDHG_TUNE_KNOBS || value < 0) return SPDHG_ERR_ARG;
   switch (knob) {
     case SPDHG_TUNE_PRIOR_COLS:
-      // the launch checks cols against the warps of a column at the current voxels per thread
+      // the launch checks cols against the warps of a column
       if (value != 0 && (value < 2 || value > 32)) return fail(ctx, SPDHG_ERR_ARG, "prior cols out of range");
       break;
     case SPDHG_TUNE_PRIOR_VZ:

@@ -191,7 +191,7 @@ struct PriorArgs {
   float sigma, alpha, inv_p, gamma_d, eta2;
 };
 cudaError_t launch_prior(const DevGeom& g, const PriorArgs& a, cudaStream_t s);
-// whether the prior kernel's launch-shape knobs fit together (voxels per thread, columns, rows)
+// whether the prior kernel's launch-shape knobs fit together
 bool prior_launch_ok(const DevGeom& g, int kind);
 
 struct TgvArgs {
@@ -202,9 +202,7 @@ struct TgvArgs {
   float* zu; float* zw;
   const float* Tu; float Tw;
   float sigma, alpha, inv_p;
-  float* bscr;                          // scratch: the dual change b (3N or 6N)
 };
-// the block's dual pass and primal pass (two kernels)
 cudaError_t launch_tgv(const DevGeom& g, const TgvArgs& a, cudaStream_t s);
 // data iteration for TGV also steps w: w -= Tw * zbar_w with zbar_w = zw (no new w-dual change)
 cudaError_t launch_w_step(const DevGeom& g, float* w, const float* zw, float Tw, cudaStream_t s);
@@ -293,7 +291,6 @@ struct spdhg_ctx {
   int wcur = 0;
   float* zw = nullptr;
   float* q2[2] = {nullptr, nullptr};
-  float* tgv_b = nullptr;      // TGV dual change of the current prior block (6N)
   int q2cur = 0;
   float Tw = 0.f;
   // scratch

@@ -136,16 +136,11 @@ extern "C" int spdhg_autotune(spdhg_ctx* ctx, int reps, int* chosen, void* strea
     knobs.push_back(k);
   }
   if (stencil) {
-    Knob vz{SPDHG_TUNE_PRIOR_VZ, false, {1, 2, 4}};
-    knobs.push_back(vz);
-    // columns per block: the launch admits cols x (warps per column) <= 32 at the chosen voxels
-    // per thread; candidates that do not fit are skipped below
+    // columns per block: candidates that do not fit the block's warps are skipped below
     Knob c{SPDHG_TUNE_PRIOR_COLS, false, {}};
     for (int v : {2, 3, 4, 6, 8, 12, 16, 32})
       if (v <= g.nx + 1) c.values.push_back(v);
     knobs.push_back(c);
-    Knob st{SPDHG_TUNE_PRIOR_STAGES, false, {3, 4}};
-    knobs.push_back(st);
     Knob y{SPDHG_TUNE_PRIOR_YCHUNK, false, {}};
     for (int v : {16, 32, 64, 128, 256})
       if (v / 2 < g.ny) y.values.push_back(v);
