@@ -1,0 +1,477 @@
+// 3x3x3 convolutions of the learned warm start (forward, data gradient, weight gradient) on the tensor
+// cores (tcgen05, BF16 x BF16 -> FP32 in TMEM) without an im2col gather.
+//
+// A tile is 16 consecutive x positions x 8 consecutive z slices at one y: 128 voxels, row r = 8 m + j
+// <-> voxel (y, x0 + m, z0 + j).  Its input halo (3 y x 18 x x 10 z voxels, zero outside the volume) is
+// staged by 8-channel groups, voxel (dy, xx, zz) of a group at ((dy * 18 + xx) * 10 + zz) * 16 bytes
+// or, for the kernels that take whole dy planes, at (xx * 10 + zz) * 16 of plane (dy, group).  For tap
+// (dy, dx, dz) the operand of the MMA is the same halo read from a shifted start: the z-run at x0 + m is
+// one core matrix (8 voxels x 16 bytes), consecutive runs are 160 bytes apart.  So a tap costs no copies.
+//
+// Bound: the MMAs' reads of the 128 x 16 operand from shared memory (about 70 cycles a step at 16 output
+// channels, where the step's products take 4), then the halo copies; so blocks are persistent, three
+// halos are in flight, and the accumulator of one tile is read while the next tile's MMAs run.  Measured
+// on GB300, 128 x 128 x 64 voxels: 32 -> 16 channels 202 -> 146 us, 16 -> 16 104 -> 58 us, 8 -> 16 101 -> 45 us
+// (from the gather); 64 -> 32 at 64 x 64 x 32 165 -> 70 us, 128 -> 128 at 16 x 16 x 8 88 -> 23 us (gather);
+// weight gradients 32 -> 16 658 -> 186 us, 16 -> 16 308 -> 108 us, 128 -> 64 174 -> 62 us (gather).  Inference
+// 1411 -> 804 us, gradients of a mini-batch of four 21.98 -> 11.91 ms.  128 threads: 897 us and 13.8 ms;
+// 512: 884 us and 12.8 ms.
+// Included by igemm.cu, whose error flag and mode table it shares.
+#pragma once
+
+namespace spdhg {
+namespace ig {
+
+constexpr int HX = 18, HZ = 10, HPL = HX * HZ, HROWS = 3 * HPL;  // halo voxels: x, z, per dy plane, in all
+constexpr int CTHREADS = 384;    // three warps per TMEM lane quarter: thread t reads lane t % 128
+constexpr int CPARTS = CTHREADS / 128;
+constexpr long long CWAIT = 4000000000ll;  // ~2 s at 2 GHz: a lost completion ends the kernel
+
+struct Tile {
+  int y, x0, z0;
+};
+__device__ __forceinline__ Tile tile_of(int t, const GemmArgs& g) {
+  const int tz = (g.nz + 7) >> 3, tx = (g.nx + 15) >> 4;
+  Tile r;
+  const int q = t / tz;
+  r.z0 = (t - q * tz) * 8;
+  r.y = q / tx;
+  r.x0 = (q - r.y * tx) * 16;
+  return r;
+}
+
+// Byte offset of tap (dy, dx, dz)'s first core matrix in a halo of whole groups.
+__host__ __device__ constexpr uint32_t tap_off(int tap) {
+  return (uint32_t)(((tap / 9) * HX + (tap / 3) % 3) * HZ + tap % 3) * 16u;
+}
+
+__device__ __forceinline__ void drain_failed(int code) {
+  set_error(code);
+  // give MMAs that may still be in flight a bounded chance to finish before TMEM is released
+  const long long t0 = clock64();
+  while (clock64() - t0 < 2000000ll) {
+  }
+}
+
+// Epilogue of one tile: thread t holds row t % 128 (TMEM lane) and every CPARTS-th group of eight of the
+// Nt columns from n_first on; tmem is the accumulator.
+__device__ __forceinline__ void conv_epilogue(const GemmArgs& g, const Tile& T, uint32_t tmem, int n_first, int Nt, const float* bias) {
+  const int row = threadIdx.x & 127, x = T.x0 + (row >> 3), z = T.z0 + (row & 7);
+  const uint32_t trow = tmem + ((uint32_t)(row & ~31) << 16);
+  const bool ok = x < g.nx && z < g.nz;
+  const size_t orow = ((size_t)T.y * g.nx + x) * g.nz + z;
+  for (int n0 = 8 * (threadIdx.x >> 7); n0 < Nt; n0 += 8 * CPARTS) {
+    float v[8];
+    umma::tmem_ld8(trow + n0, v);
+    if (!ok) continue;
+    const int n = n_first + n0;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      v[j] += bias[n0 + j];
+      if (g.relu) v[j] = fmaxf(v[j], 0.f);
+    }
+    if (g.mask && n + 8 > g.mask_from) {
+      const uint4 mk = *reinterpret_cast<const uint4*>(g.mask + orow * g.mask_stride + g.mask_off + n);
+      const __nv_bfloat162* m2 = reinterpret_cast<const __nv_bfloat162*>(&mk);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const float2 f = __bfloat1622float2(m2[j]);
+        if (n + 2 * j >= g.mask_from && !(f.x > 0.f)) v[2 * j] = 0.f;
+        if (n + 2 * j + 1 >= g.mask_from && !(f.y > 0.f)) v[2 * j + 1] = 0.f;
+      }
+    }
+    __align__(16) __nv_bfloat162 h[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) h[j] = __floats2bfloat162_rn(v[2 * j], v[2 * j + 1]);
+    *reinterpret_cast<uint4*>(g.out + orow * g.out_stride + g.out_off + n) = *reinterpret_cast<uint4*>(h);
+  }
+}
+
+__device__ __forceinline__ void load_bias(const GemmArgs& g, int n_first, int Nt, float* sbias) {
+  if ((int)threadIdx.x < Nt) sbias[threadIdx.x] = g.bias ? g.bias[n_first + threadIdx.x] : 0.f;
+}
+
+// ------------------------------------------------------------------------------------------
+// up to 32 input channels: persistent blocks, all weights of an N slice resident, three halo buffers
+// ------------------------------------------------------------------------------------------
+
+constexpr int kHaloBufs = 3;
+
+template <int C>
+__global__ void __launch_bounds__(CTHREADS) k_conv3_halo(const __grid_constant__ GemmArgs g, int tiles, int Nt) {
+  constexpr int CG = C / 8;                            // channel groups
+  constexpr uint32_t GP = HROWS * 16;                  // bytes of a group's halo
+  constexpr int PIECES = (HROWS * CG + CTHREADS - 1) / CTHREADS;
+  constexpr int TAPS = C == 8 ? 28 : 27;               // weight blocks (8 channels: taps 0 .. 25, zeros, tap 26)
+  extern __shared__ __align__(1024) unsigned char smem[];
+  __shared__ uint64_t mbar[2];
+  __shared__ uint32_t tmem_slot;
+  __shared__ float sbias[32];
+  const int tid = threadIdx.x, warp = tid >> 5, n_first = blockIdx.y * Nt;
+  const uint32_t sh = umma::smem_u32(smem), halo = CG * GP, sb = sh + kHaloBufs * halo;
+  const uint32_t tapb = (uint32_t)(Nt >> 3) * CG * 128;  // bytes of a tap's weights (this slice)
+  uint32_t ncols = 32;
+  while ((int)ncols < 2 * Nt) ncols <<= 1;
+  if (warp == 0) umma::tmem_alloc(&tmem_slot, ncols);
+  if (tid == 0) {
+    umma::mbar_init(&mbar[0], 1);
+    umma::mbar_init(&mbar[1], 1);
+    umma::fence_mbar_init();
+  }
+  load_bias(g, n_first, Nt, sbias);
+  // weights: [tap][n / 8][c / 8] core matrices; the slice's rows of a tap are contiguous
+  for (int i = tid; i < TAPS * (int)(tapb >> 4); i += CTHREADS) {
+    const int tap = i / (int)(tapb >> 4), k = i - tap * (int)(tapb >> 4);
+    umma::cp16(sb + 16 * i, g.b + ((size_t)tap * g.N + n_first) * C + 8 * k, 16u);
+  }
+  // this thread's pieces of a halo: (dy, xx, zz, group), groups fastest (32 contiguous bytes per voxel pair)
+  auto stage = [&](int t, int buf) {
+    const Tile T = tile_of(t, g);
+    const __nv_bfloat16* base = g.a + g.a_off;
+#pragma unroll 4
+    for (int k = 0; k < PIECES; ++k) {
+      const int idx = tid + CTHREADS * k;
+      if (idx >= HROWS * CG) break;
+      const int cg = idx % CG, h = idx / CG, dy = h / HPL, rem = h - dy * HPL, xx = rem / HZ, zz = rem - xx * HZ;
+      const int yy = T.y + dy - 1, xg = T.x0 + xx - 1, zg = T.z0 + zz - 1;
+      const bool ok = (unsigned)yy < (unsigned)g.ny && (unsigned)xg < (unsigned)g.nx && (unsigned)zg < (unsigned)g.nz;
+      const __nv_bfloat16* src = ok ? base + ((size_t)(yy * g.nx + xg) * g.nz + zg) * g.a_stride + cg * 8 : g.a;
+      umma::cp16(sh + buf * halo + cg * GP + h * 16, src, ok ? 16u : 0u);
+    }
+  };
+  const int n = blockIdx.x < tiles ? (tiles - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
+  auto tile_at = [&](int it) { return blockIdx.x + it * gridDim.x; };
+  if (n > 0) stage(tile_at(0), 0);
+  umma::cp_commit();  // the weights too
+  if (n > 1) stage(tile_at(1), 1);
+  umma::cp_commit();
+  umma::fence_before_sync();
+  __syncthreads();
+  umma::fence_after_sync();
+  const uint32_t tmem = tmem_slot;
+  const uint32_t idesc = umma::idesc_bf16(128, Nt, false, false);
+  bool failed = false;
+  for (int it = 0; it < n; ++it) {
+    umma::cp_wait<1>();  // tile `it` has landed (this thread's copies)
+    umma::fence_proxy_async_smem();
+    umma::fence_before_sync();
+    if (__syncthreads_or(failed)) break;
+    if (tid == 0) {
+      umma::fence_after_sync();
+      const uint32_t a0 = sh + (it % kHaloBufs) * halo, d = tmem + (it & 1) * Nt;
+      if (C == 8) {
+        // a K step holds two taps; the distance of their starts is the leading-dimension offset.  The
+        // last step pairs tap 26 with tap 25 under zero weights (no read leaves the halo)
+#pragma unroll
+        for (int i = 0; i < 14; ++i) {
+          const int t0 = i < 13 ? 2 * i : 25, t1 = i < 13 ? 2 * i + 1 : 26;
+          umma::mma_bf16(d, umma::smem_desc(a0 + tap_off(t0), tap_off(t1) - tap_off(t0), HZ * 16),
+                         umma::smem_desc(sb + 2 * i * tapb, tapb, 128), idesc, i > 0 ? 1u : 0u);
+        }
+      } else {
+#pragma unroll
+        for (int tap = 0; tap < 27; ++tap)
+#pragma unroll
+          for (int c16 = 0; c16 < C / 16; ++c16)
+            umma::mma_bf16(d, umma::smem_desc(a0 + 2 * c16 * GP + tap_off(tap), GP, HZ * 16),
+                           umma::smem_desc(sb + tap * tapb + 2 * c16 * 128, 128, CG * 128), idesc, tap + c16 > 0 ? 1u : 0u);
+      }
+      umma::commit(&mbar[it & 1]);
+    }
+    if (it > 0) {
+      // the previous tile's accumulator, while this tile's MMAs run; its halo buffer is free then
+      failed = __any_sync(0xffffffffu, !umma::mbar_wait(&mbar[(it - 1) & 1], ((it - 1) >> 1) & 1, CWAIT));
+      umma::fence_after_sync();
+      if (!failed) conv_epilogue(g, tile_of(tile_at(it - 1), g), tmem + ((it - 1) & 1) * Nt, n_first, Nt, sbias);
+    }
+    if (!failed && it + 2 < n) stage(tile_at(it + 2), (it + 2) % kHaloBufs);
+    umma::cp_commit();
+  }
+  umma::cp_wait<0>();
+  if (n > 0 && !failed) {
+    failed = __any_sync(0xffffffffu, !umma::mbar_wait(&mbar[(n - 1) & 1], ((n - 1) >> 1) & 1, CWAIT));
+    umma::fence_after_sync();
+    if (!failed) conv_epilogue(g, tile_of(tile_at(n - 1), g), tmem + ((n - 1) & 1) * Nt, n_first, Nt, sbias);
+  }
+  if (__syncthreads_or(failed)) drain_failed(2);
+  umma::fence_before_sync();
+  __syncthreads();
+  if (warp == 0) umma::tmem_dealloc(tmem, ncols);
+}
+
+// ------------------------------------------------------------------------------------------
+// 64 and 128 input channels: one tile and N slice per block, the halo's dy planes resident, the
+// weights streamed tap by tap (bulk copies, four in flight)
+// ------------------------------------------------------------------------------------------
+
+constexpr int kTapRing = 4;
+
+template <int C>
+__global__ void __launch_bounds__(CTHREADS) k_conv3_deep(const __grid_constant__ GemmArgs g, int Nt) {
+  constexpr int CG = C / 8;
+  constexpr uint32_t GP = HPL * 16, DY = CG * GP;      // bytes of a (dy, group) plane and of a dy plane
+  extern __shared__ __align__(1024) unsigned char smem[];
+  __shared__ uint64_t full[kTapRing], empty[kTapRing], done;
+  __shared__ uint32_t tmem_slot;
+  __shared__ float sbias[32];
+  const int tid = threadIdx.x, warp = tid >> 5, n_first = blockIdx.y * Nt;
+  const uint32_t sh = umma::smem_u32(smem), sb = sh + 3 * DY;
+  const uint32_t tapb = (uint32_t)Nt * C * 2;
+  if (warp == 0) umma::tmem_alloc(&tmem_slot, 32);
+  if (tid == 0) {
+    for (int k = 0; k < kTapRing; ++k) {
+      umma::mbar_init(&full[k], 1);
+      umma::mbar_init(&empty[k], 1);
+    }
+    umma::mbar_init(&done, 1);
+    umma::fence_mbar_init();
+  }
+  load_bias(g, n_first, Nt, sbias);
+  umma::fence_before_sync();
+  __syncthreads();
+  umma::fence_after_sync();
+  auto load_tap = [&](int tap) {
+    const int s = tap % kTapRing;
+    umma::bulk_load(sb + s * tapb, g.b + ((size_t)tap * g.N + n_first) * C, tapb, &full[s]);
+  };
+  if (tid == 0)
+    for (int tap = 0; tap < kTapRing; ++tap) load_tap(tap);
+  const Tile T = tile_of(blockIdx.x, g);
+  for (int dy = 0; dy < 3; ++dy) {
+    const int yy = T.y + dy - 1;
+    for (int idx = tid; idx < HPL * CG; idx += CTHREADS) {
+      const int cg = idx % CG, h = idx / CG, xx = h / HZ, zz = h - xx * HZ;
+      const int xg = T.x0 + xx - 1, zg = T.z0 + zz - 1;
+      const bool ok = (unsigned)yy < (unsigned)g.ny && (unsigned)xg < (unsigned)g.nx && (unsigned)zg < (unsigned)g.nz;
+      const __nv_bfloat16* src = ok ? g.a + g.a_off + ((size_t)(yy * g.nx + xg) * g.nz + zg) * g.a_stride + cg * 8 : g.a;
+      umma::cp16(sh + dy * DY + cg * GP + h * 16, src, ok ? 16u : 0u);
+    }
+    umma::cp_commit();
+  }
+  const uint32_t tmem = tmem_slot, idesc = umma::idesc_bf16(128, Nt, false, false);
+  bool failed = false;
+  for (int dy = 0; dy < 3; ++dy) {
+    if (dy == 0) umma::cp_wait<2>();
+    else if (dy == 1) umma::cp_wait<1>();
+    else umma::cp_wait<0>();
+    umma::fence_proxy_async_smem();
+    __syncthreads();
+    if (tid == 0) {
+      for (int k = 0; k < 9 && !failed; ++k) {
+        const int tap = 9 * dy + k, s = tap % kTapRing;
+        failed = !umma::mbar_wait(&full[s], (tap / kTapRing) & 1, CWAIT);
+        if (failed) break;
+        umma::fence_after_sync();
+        const uint32_t a0 = sh + dy * DY + (uint32_t)((k / 3) * HZ + k % 3) * 16, b0 = sb + s * tapb;
+        for (int c16 = 0; c16 < C / 16; ++c16)
+          umma::mma_bf16(tmem, umma::smem_desc(a0 + 2 * c16 * GP, GP, HZ * 16), umma::smem_desc(b0 + 2 * c16 * 128, 128, CG * 128),
+                         idesc, tap + c16 > 0 ? 1u : 0u);
+        umma::commit(&empty[s]);
+        if (tap > 0 && tap - 1 + kTapRing < 27) {  // the slot of the previous tap, once its MMAs are done
+          failed = !umma::mbar_wait(&empty[(tap - 1) % kTapRing], ((tap - 1) / kTapRing) & 1, CWAIT);
+          if (!failed) load_tap(tap - 1 + kTapRing);
+        }
+      }
+      if (dy == 2) umma::commit(&done);
+    }
+  }
+  failed = !umma::mbar_wait(&done, 0, CWAIT) || failed;
+  const bool any = __syncthreads_or(failed);
+  if (any) drain_failed(3);
+  umma::fence_after_sync();
+  if (!any) conv_epilogue(g, T, tmem, n_first, Nt, sbias);
+  umma::fence_before_sync();
+  __syncthreads();
+  if (warp == 0) umma::tmem_dealloc(tmem, 32);
+}
+
+cudaError_t launch_conv3(const GemmArgs& g, cudaStream_t s) {
+  const int C = g.a_c, Nt = std::min(32, g.N);
+  if ((C != 8 && C != 16 && C != 32 && C != 64 && C != 128) || (g.N != 16 && g.N % 32)) return cudaErrorNotSupported;
+  const int tiles = ((g.nz + 7) / 8) * ((g.nx + 15) / 16) * g.ny;
+  auto go = [&](auto kern, dim3 grid, size_t smem, auto... args) -> cudaError_t {
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    kern<<<grid, CTHREADS, smem, s>>>(g, args...);
+    return cudaGetLastError();
+  };
+  if (C <= 32) {
+    const size_t smem = (size_t)kHaloBufs * (C / 8) * HROWS * 16 + (size_t)(C == 8 ? 28 : 27) * Nt * C * 2;
+    const int per_sm = std::max(1, std::min(4, (int)(220 * 1024 / (smem + 1024)))), slices = g.N / Nt;
+    const dim3 grid(std::min(tiles, std::max(1, 152 * per_sm / slices)), slices);
+    if (C == 8) return go(k_conv3_halo<8>, grid, smem, tiles, Nt);
+    if (C == 16) return go(k_conv3_halo<16>, grid, smem, tiles, Nt);
+    return go(k_conv3_halo<32>, grid, smem, tiles, Nt);
+  }
+  const size_t smem = (size_t)3 * (C / 8) * HPL * 16 + (size_t)kTapRing * Nt * C * 2;
+  const dim3 grid(tiles, g.N / Nt);
+  if (C == 64) return go(k_conv3_deep<64>, grid, smem, Nt);
+  return go(k_conv3_deep<128>, grid, smem, Nt);
+}
+
+// ------------------------------------------------------------------------------------------
+// weight gradient: D[(tap, ci)][co] = sum over voxels v of in[v + tap][ci] g[v][co]
+//
+// The reduction runs over the tile's voxels, so both operands are MN-major: a core matrix is a z-run
+// of 8 voxels x 8 channels, the same bytes as above.  The halo is laid out by planes (dy, group), all
+// of one size, so the M blocks of one (dx, dz) are the planes in order: rows (dy, ci) of three taps at
+// once, 3 C rows in M = 128 chunks, and a plane of ones after them whose rows sum the columns of g (the
+// bias gradient).  The nine (dx, dz) accumulators stay in TMEM over all tiles of a persistent block; its
+// partial sums are then reduced over the blocks in a fixed order.
+// ------------------------------------------------------------------------------------------
+
+template <int C>
+struct Wg {
+  static constexpr int CG = C / 8, PLANES = 3 * CG;
+  static constexpr int CHUNKS = (3 * C + 127) / 128;           // M = 128 chunks
+  static constexpr bool ONES = 3 * C < CHUNKS * 128;           // a spare plane for the bias gradient
+  static constexpr int BUFS = C <= 32 ? 3 : (C == 64 ? 2 : 1);
+  static constexpr uint32_t GP = HPL * 16;                     // bytes of a plane
+  static constexpr uint32_t ABYTES = (PLANES + (ONES ? 1 : 0)) * GP;
+};
+
+template <int C>
+__global__ void __launch_bounds__(CTHREADS) k_wgrad3(const __grid_constant__ GemmArgs g, int tiles, int Nt, float* bias_part) {
+  using W = Wg<C>;
+  constexpr int CG = W::CG, BUFS = W::BUFS;
+  constexpr uint32_t GP = W::GP;
+  extern __shared__ __align__(1024) unsigned char smem[];
+  __shared__ uint64_t mbar[BUFS];
+  __shared__ uint32_t tmem_slot;
+  const int tid = threadIdx.x, warp = tid >> 5, n_first = blockIdx.y * Nt, NG = Nt >> 3;
+  const uint32_t sh = umma::smem_u32(smem), bbytes = (uint32_t)NG * 2048, buf_bytes = W::ABYTES + bbytes;
+  uint32_t ncols = 32;
+  while ((int)ncols < 9 * Nt * W::CHUNKS) ncols <<= 1;
+  if (warp == 0) umma::tmem_alloc(&tmem_slot, ncols);
+  if (tid == 0) {
+    for (int k = 0; k < BUFS; ++k) umma::mbar_init(&mbar[k], 1);
+    umma::fence_mbar_init();
+  }
+  if (W::ONES) {  // one in the first channel of every voxel
+    for (int i = tid; i < BUFS * HPL; i += CTHREADS) {
+      const int k = i / HPL, h = i - k * HPL;
+      *reinterpret_cast<uint4*>(smem + k * buf_bytes + W::PLANES * GP + h * 16) = make_uint4(0x3F80u, 0u, 0u, 0u);
+    }
+  }
+  auto stage = [&](int t, int buf) {
+    const Tile T = tile_of(t, g);
+    const uint32_t sa = sh + buf * buf_bytes, sg = sa + W::ABYTES;
+    for (int idx = tid; idx < HROWS * CG; idx += CTHREADS) {
+      const int cg = idx % CG, h = idx / CG, dy = h / HPL, rem = h - dy * HPL, xx = rem / HZ, zz = rem - xx * HZ;
+      const int yy = T.y + dy - 1, xg = T.x0 + xx - 1, zg = T.z0 + zz - 1;
+      const bool ok = (unsigned)yy < (unsigned)g.ny && (unsigned)xg < (unsigned)g.nx && (unsigned)zg < (unsigned)g.nz;
+      const __nv_bfloat16* src = ok ? g.a + g.a_off + ((size_t)(yy * g.nx + xg) * g.nz + zg) * g.a_stride + cg * 8 : g.a;
+      umma::cp16(sa + (dy * CG + cg) * GP + rem * 16, src, ok ? 16u : 0u);
+    }
+    for (int idx = tid; idx < 128 * NG; idx += CTHREADS) {
+      const int ng = idx % NG, r = idx / NG, x = T.x0 + (r >> 3), z = T.z0 + (r & 7);
+      const bool ok = x < g.nx && z < g.nz;
+      const __nv_bfloat16* src = ok ? g.b + g.b_off + ((size_t)(T.y * g.nx + x) * g.nz + z) * g.b_stride + n_first + ng * 8 : g.b;
+      umma::cp16(sg + ng * 2048 + r * 16, src, ok ? 16u : 0u);
+    }
+  };
+  const int n = blockIdx.x < tiles ? (tiles - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
+  auto tile_at = [&](int it) { return blockIdx.x + it * gridDim.x; };
+  for (int k = 0; k < std::max(1, BUFS - 1); ++k) {
+    if (k < n) stage(tile_at(k), k);
+    umma::cp_commit();
+  }
+  umma::fence_before_sync();
+  __syncthreads();
+  umma::fence_after_sync();
+  const uint32_t tmem = tmem_slot;
+  const uint32_t idesc = umma::idesc_bf16(128, Nt, true, true);
+  bool failed = false;
+  for (int it = 0; it < n; ++it) {
+    umma::cp_wait<(BUFS > 2 ? BUFS - 2 : 0)>();
+    umma::fence_proxy_async_smem();
+    if (__syncthreads_or(failed)) break;
+    if (tid == 0) {
+      umma::fence_after_sync();
+      const uint32_t sa = sh + (it % BUFS) * buf_bytes, sg = sa + W::ABYTES;
+      for (int t9 = 0; t9 < 9; ++t9) {
+        const uint32_t a0 = sa + (uint32_t)((t9 / 3) * HZ + t9 % 3) * 16;
+#pragma unroll
+        for (int ch = 0; ch < W::CHUNKS; ++ch)
+#pragma unroll
+          for (int ks = 0; ks < 8; ++ks)  // 16 voxels: two z-runs
+            umma::mma_bf16(tmem + (t9 * W::CHUNKS + ch) * Nt, umma::smem_desc(a0 + ch * 16 * GP + ks * 2 * HZ * 16, HZ * 16, GP),
+                           umma::smem_desc(sg + ks * 256, 128, 2048), idesc, it + ks > 0 ? 1u : 0u);
+      }
+      umma::commit(&mbar[it % BUFS]);
+    }
+    const int nx = it + std::max(1, BUFS - 1);
+    if (nx < n) {
+      // the buffer of tile nx was last read by the MMAs of tile nx - BUFS
+      const int prev = nx - BUFS;
+      if (prev >= 0) failed = !umma::mbar_wait(&mbar[prev % BUFS], (prev / BUFS) & 1, CWAIT);
+      if (!failed) stage(tile_at(nx), nx % BUFS);
+    }
+    umma::cp_commit();
+  }
+  umma::cp_wait<0>();
+  if (n > 0 && !failed) failed = !umma::mbar_wait(&mbar[(n - 1) % BUFS], ((n - 1) / BUFS) & 1, CWAIT);
+  const bool any = __syncthreads_or(failed);
+  if (any) drain_failed(4);
+  umma::fence_after_sync();
+  // partial sums: row m of chunk ch is (dy, ci) = ((128 ch + m) / C, (128 ch + m) % C)
+  const uint32_t trow = tmem + ((uint32_t)(tid & 96) << 16);
+  for (int ch = 0; ch < W::CHUNKS; ++ch) {
+    const int m = ch * 128 + (tid & 127), dy = m / C, ci = m - dy * C;
+    for (int t9 = tid >> 7; t9 < 9; t9 += CPARTS)
+      for (int n0 = 0; n0 < Nt; n0 += 8) {
+        float v[8];
+        umma::tmem_ld8(trow + (t9 * W::CHUNKS + ch) * Nt + n0, v);
+        if (any) continue;
+        float* dst = nullptr;
+        if (m < 3 * C) dst = g.outf + ((size_t)blockIdx.x * 27 * C + (size_t)(dy * 9 + t9) * C + ci) * g.N + n_first + n0;
+        else if (W::ONES && m == 3 * C && t9 == 0) dst = bias_part + (size_t)blockIdx.x * g.N + n_first + n0;
+        if (!dst) continue;
+        *reinterpret_cast<float4*>(dst) = n > 0 ? make_float4(v[0], v[1], v[2], v[3]) : make_float4(0.f, 0.f, 0.f, 0.f);
+        *reinterpret_cast<float4*>(dst + 4) = n > 0 ? make_float4(v[4], v[5], v[6], v[7]) : make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+  }
+  umma::fence_before_sync();
+  __syncthreads();
+  if (warp == 0) umma::tmem_dealloc(tmem, ncols);
+}
+
+static int wgrad_slice(int C, int N) { return C <= 32 ? std::min(32, N) : 16; }
+
+int wgrad3_blocks(const GemmArgs& g) {
+  const int tiles = ((g.nz + 7) / 8) * ((g.nx + 15) / 16) * g.ny, slices = g.N / wgrad_slice(g.a_c, g.N);
+  return std::min(tiles, std::max(1, 152 * (g.a_c <= 16 ? 2 : 1) / slices));
+}
+
+bool wgrad3_fits(const GemmArgs& g) {
+  const int C = g.a_c;
+  return (C == 8 || C == 16 || C == 32 || C == 64 || C == 128) && (g.N == 16 || g.N % 32 == 0);
+}
+
+bool wgrad3_sums_bias(int C) { return C < 128; }
+
+cudaError_t launch_wgrad3(const GemmArgs& g, float* bias_part, cudaStream_t s) {
+  if (!wgrad3_fits(g)) return cudaErrorNotSupported;
+  const int C = g.a_c, Nt = wgrad_slice(C, g.N);
+  const int tiles = ((g.nz + 7) / 8) * ((g.nx + 15) / 16) * g.ny;
+  const dim3 grid(wgrad3_blocks(g), g.N / Nt);
+  auto go = [&](auto kern, size_t abytes, int bufs, int chunks) -> cudaError_t {
+    // the last chunk's M blocks may run past the planes: their rows are not used, but must be readable
+    const size_t reach = (size_t)chunks * 16 * HPL * 16 + 2 * HZ * 16 + 1024;
+    const size_t smem = (size_t)(bufs - 1) * (abytes + (size_t)(Nt / 8) * 2048) + std::max(abytes + (size_t)(Nt / 8) * 2048, reach);
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    kern<<<grid, CTHREADS, smem, s>>>(g, tiles, Nt, bias_part);
+    return cudaGetLastError();
+  };
+  switch (C) {
+    case 8: return go(k_wgrad3<8>, Wg<8>::ABYTES, Wg<8>::BUFS, Wg<8>::CHUNKS);
+    case 16: return go(k_wgrad3<16>, Wg<16>::ABYTES, Wg<16>::BUFS, Wg<16>::CHUNKS);
+    case 32: return go(k_wgrad3<32>, Wg<32>::ABYTES, Wg<32>::BUFS, Wg<32>::CHUNKS);
+    case 64: return go(k_wgrad3<64>, Wg<64>::ABYTES, Wg<64>::BUFS, Wg<64>::CHUNKS);
+    default: return go(k_wgrad3<128>, Wg<128>::ABYTES, Wg<128>::BUFS, Wg<128>::CHUNKS);
+  }
+}
+
+}  // namespace ig
+}  // namespace spdhg

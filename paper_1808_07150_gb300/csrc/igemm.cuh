@@ -42,15 +42,22 @@ struct GemmArgs {
   float* outf;
   const __nv_bfloat16* mask; int mask_stride, mask_off;  // zero where mask <= 0 (ReLU gradient)
   int mask_from;               // columns below this one are not masked
-  int out_child;               // rows go to child(row, blockIdx.z) on the 2x grid
+  int out_child;               // transposed convolution: channels c per child; column n goes to channel n % c
+                               // of child (blockIdx.z N / c + n / c) of the row's voxel on the 2x grid (0: no)
   int k_per_split;             // E_PART: reduction elements per blockIdx.y (multiple of 64)
 };
 
 cudaError_t launch(int am, int bm, int em, const GemmArgs& g, dim3 grid, cudaStream_t s);
-// 3x3x3 convolution (A_CONV3 operands, B = weights [N][27 a_c]) from a staged input halo with the
-// taps as shifted shared-memory descriptors; cudaErrorNotSupported when the shape does not fit
-// (a_c in {16, 32}, N <= 64, nx % 16 == 0, nz % 8 == 0), in which case launch() serves it
-cudaError_t launch_conv3_halo(int em, const GemmArgs& g, cudaStream_t s);
+// 3x3x3 convolution (A_CONV3 operands; B = weights [tap][N / 8][a_c / 8][8][8], a zero
+// block before tap 26 for a_c = 8) from a staged input halo with the taps as shifted shared-memory descriptors, BF16 output;
+// cudaErrorNotSupported for 256 input channels, which launch() serves with weights [N][27 a_c]
+cudaError_t launch_conv3(const GemmArgs& g, cudaStream_t s);
+// 3x3x3 weight gradient (A_WG_CONV3, B_WG_ROWS operands): partial sums outf[block][27 a_c][N] of
+// wgrad3_blocks(g) blocks, and the column sums of b in bias_part[block][N] where wgrad3_sums_bias(a_c)
+bool wgrad3_fits(const GemmArgs& g);
+bool wgrad3_sums_bias(int a_c);
+int wgrad3_blocks(const GemmArgs& g);
+cudaError_t launch_wgrad3(const GemmArgs& g, float* bias_part, cudaStream_t s);
 // first failure code recorded by any launch (0: none); synchronises s
 int read_error(cudaStream_t s);
 

@@ -19,6 +19,7 @@
 #include <stdint.h>
 #include <string.h>
 
+#include <algorithm>
 #include <string>
 #include <vector>
 
@@ -100,7 +101,15 @@ __global__ void k_head_fwd(const bf16* __restrict__ h, int C, const float* __res
                            const float* __restrict__ xn, float* __restrict__ pred, int64_t V) {
   for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < V; v += (int64_t)gridDim.x * blockDim.x) {
     float a = xn[v] + b[0];
-    for (int c = 0; c < C; ++c) a = fmaf(w[c], __bfloat162float(h[v * C + c]), a);
+    for (int c = 0; c < C; c += 8) {
+      const uint4 q = *reinterpret_cast<const uint4*>(h + v * C + c);
+      const __nv_bfloat162* q2 = reinterpret_cast<const __nv_bfloat162*>(&q);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const float2 f = __bfloat1622float2(q2[k]);
+        a = fmaf(w[c + 2 * k + 1], f.y, fmaf(w[c + 2 * k], f.x, a));
+      }
+    }
     pred[v] = a;
   }
 }
@@ -129,11 +138,20 @@ __global__ void k_mse(const float* __restrict__ pred, const float* __restrict__ 
 // gradient of the pre-activation of the last decoder conv: w_c gpred (h_c > 0)
 __global__ void k_head_bwd(const float* __restrict__ gpred, const bf16* __restrict__ h, int C, const float* __restrict__ w,
                            bf16* __restrict__ gh, int64_t V) {
-  const int64_t n = V * C;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const int c = (int)(i % C);
-    const int64_t v = i / C;
-    gh[i] = __float2bfloat16_rn(__bfloat162float(h[i]) > 0.f ? w[c] * gpred[v] : 0.f);
+  const int groups = C >> 3;  // eight channels (16 bytes) a thread
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < V * groups; i += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t v = groups == 2 ? i >> 1 : i / groups;
+    const int c = (int)(i - v * groups) * 8;
+    const float gp = gpred[v];
+    const uint4 q = *reinterpret_cast<const uint4*>(h + 8 * i);
+    const __nv_bfloat162* q2 = reinterpret_cast<const __nv_bfloat162*>(&q);
+    __align__(16) __nv_bfloat162 o[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const float2 f = __bfloat1622float2(q2[k]);
+      o[k] = __floats2bfloat162_rn(f.x > 0.f ? w[c + 2 * k] * gp : 0.f, f.y > 0.f ? w[c + 2 * k + 1] * gp : 0.f);
+    }
+    *reinterpret_cast<uint4*>(gh + 8 * i) = *reinterpret_cast<uint4*>(o);
   }
 }
 
@@ -194,6 +212,26 @@ __global__ void k_wg_conv3(const float* __restrict__ part, int splits, int cin, 
   }
 }
 
+// the same from the blocks of launch_wgrad3, whose many partial sums four threads per element share:
+// 64 elements x 4 split residues per block, added in a fixed order
+__global__ void __launch_bounds__(256) k_wg_reduce(const float* __restrict__ part, int splits, int cin, int cout,
+                                                   float* __restrict__ g, int accumulate) {
+  __shared__ float sh[4][64];
+  const int n = 27 * cin * cout, e = threadIdx.x & 63, q = threadIdx.x >> 6, i = blockIdx.x * 64 + e;
+  float s = 0.f;
+  if (i < n) {
+#pragma unroll 8
+    for (int k = q; k < splits; k += 4) s += part[(size_t)k * n + i];
+  }
+  sh[q][e] = s;
+  __syncthreads();
+  if (q > 0 || i >= n) return;
+  s = (sh[0][e] + sh[1][e]) + (sh[2][e] + sh[3][e]);
+  const int co = i % cout, m = i / cout, tap = m / cin, ci = m % cin;  // m = tap * cin + ci
+  float* d = g + ((size_t)co * 27 + tap) * cin + ci;
+  *d = accumulate ? *d + s : s;
+}
+
 // tconv weight gradient: part[o][split][ci][co] -> g[o][co][ci] (+)=
 __global__ void k_wg_tconv(const float* __restrict__ part, int splits, int cin, int cout, float* __restrict__ g,
                            int accumulate) {
@@ -207,14 +245,19 @@ __global__ void k_wg_tconv(const float* __restrict__ part, int splits, int cin, 
   }
 }
 
-// BF16 weight copies: conv3 forward [co][tap][ci] and flipped data-gradient [ci][tap][co]
+// position of (n, c) among the core matrices of a tap's N x C weights
+__device__ __forceinline__ int core_at(int n, int c, int C) { return ((n >> 3) * (C >> 3) + (c >> 3)) * 64 + (n & 7) * 8 + (c & 7); }
+
+// BF16 weight copies of conv3, tap by tap in core matrices: forward (N = co, C = ci) and flipped
+// data-gradient (N = ci, C = co); 256 input channels: forward [co][tap][ci]
 __global__ void k_bf16_conv3(const float* __restrict__ w, int cin, int cout, bf16* __restrict__ wf, bf16* __restrict__ wb) {
-  const int n = cout * 27 * cin;
+  const int n = cout * 27 * cin, per_tap = cin * cout;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     const int ci = i % cin, tap = (i / cin) % 27, co = i / (27 * cin);
     const bf16 h = __float2bfloat16_rn(w[i]);
-    wf[i] = h;
-    wb[((size_t)ci * 27 + (26 - tap)) * cout + co] = h;
+    const int pos = cin == 8 && tap == 26 ? 27 : tap;  // 8 channels: zeros at 26
+    wf[cin > 128 ? i : pos * per_tap + core_at(co, ci, cin)] = h;
+    wb[(26 - tap) * per_tap + core_at(ci, co, cout)] = h;
   }
 }
 
@@ -372,9 +415,9 @@ struct View {
   int stride, off, c;
 };
 
-// 3x3x3 convolution pass: the halo kernel where the shape allows it, else the gather kernel
+// 3x3x3 convolution pass: the halo kernels, or the gather kernel for 256 input channels
 int conv3_launch(unet_net* net, const ig::GemmArgs& a, cudaStream_t s) {
-  cudaError_t e = ig::launch_conv3_halo(ig::E_BF16, a, s);
+  cudaError_t e = ig::launch_conv3(a, s);
   if (e == cudaErrorNotSupported)  // returned before any CUDA call: the shape does not fit
     e = ig::launch(ig::A_CONV3, ig::B_GEMM_K, ig::E_BF16, a, dim3((a.M + 127) / 128), s);
   UCK(e);
@@ -446,6 +489,18 @@ int conv3_wgrad(unet_net* net, int l, const Param& pr, View x, View gv, int accu
   a.a = x.p; a.a_stride = x.stride; a.a_off = x.off; a.a_c = pr.cin;
   a.b = gv.p; a.b_stride = gv.stride; a.b_off = gv.off;
   a.ny = net->ny[l]; a.nx = net->nx[l]; a.nz = net->nz[l];
+  if (ig::wgrad3_fits(a)) {
+    const int nb = ig::wgrad3_blocks(a);
+    if (int st = ensure_part(net, (size_t)nb * a.M * a.N)) return st;
+    a.outf = net->part;
+    UCK(ig::launch_wgrad3(a, net->cpart, s));
+    k_wg_reduce<<<(27 * pr.cin * pr.cout + 63) / 64, 256, 0, s>>>(net->part, nb, pr.cin, pr.cout, net->g + pr.off_w, accumulate);
+    UCK(cudaGetLastError());
+    if (!ig::wgrad3_sums_bias(pr.cin)) return colsum(net, gv, net->V[l], net->g + pr.off_b, accumulate, s);
+    k_sum_parts<<<pr.cout, 256, 0, s>>>(net->cpart, nb, pr.cout, net->g + pr.off_b, accumulate);
+    UCK(cudaGetLastError());
+    return UNET_OK;
+  }
   const int tiles = (a.M + 127) / 128;
   const int splits = split_count(a.K, tiles);
   a.k_per_split = (int)(((a.K + splits - 1) / splits + 63) / 64 * 64);
@@ -462,16 +517,17 @@ int conv3_wgrad(unet_net* net, int l, const Param& pr, View x, View gv, int accu
 // transposed convolution from level l+1 (coarse) into the left half of cat[l]
 int tconv_fwd(unet_net* net, int l, const Param& pr, View x, cudaStream_t s) {
   ig::GemmArgs a{};
+  const int children = std::min(8, 256 / pr.cout);  // children per block: their weights are consecutive rows of B
   a.M = (int)net->V[l + 1];
-  a.N = pr.cout;
+  a.N = children * pr.cout;
   a.K = pr.cin;
   a.a = x.p; a.a_stride = x.stride; a.a_off = x.off; a.a_c = pr.cin;
-  a.b = pr.wf; a.b_stride = pr.cin; a.b_zstride = (long long)pr.cout * pr.cin;
+  a.b = pr.wf; a.b_stride = pr.cin; a.b_zstride = (long long)a.N * pr.cin;
   a.ny = net->ny[l + 1]; a.nx = net->nx[l + 1]; a.nz = net->nz[l + 1];
   a.bias = net->w + pr.off_b;
   a.out = net->cat[l]; a.out_stride = 2 * net->ch[l]; a.out_off = 0;
-  a.out_child = 1;
-  UCK(ig::launch(ig::A_ROWS, ig::B_GEMM_K, ig::E_BF16, a, dim3((a.M + 127) / 128, 1, 8), s));
+  a.out_child = pr.cout;
+  UCK(ig::launch(ig::A_ROWS, ig::B_GEMM_K, ig::E_BF16, a, dim3((a.M + 127) / 128, 1, 8 / children), s));
   return UNET_OK;
 }
 
@@ -605,7 +661,7 @@ int unet_create(int levels, const int* channels, int ny, int nx, int nz, unet_ne
   A(zalloc(&net->v, off));
   for (Param& p : net->P)
     if (p.kind != 2) {
-      A(zalloc(&p.wf, p.n));
+      A(zalloc(&p.wf, p.n + (p.kind == 0 ? (size_t)p.cout * p.cin : 0)));  // conv3 of 8 channels: a zero tap
       A(zalloc(&p.wb, p.n));
     }
   const int64_t V0 = net->V[0];
@@ -827,7 +883,7 @@ int unet_backward(unet_net* net, const float* target, const float* gpred_in, int
     k_sum_parts<<<c0, 256, 0, s>>>(net->cpart, kColsumBlocks, c0, net->g + hd.off_w, accumulate);
     k_colsum_part<float><<<kColsumBlocks, 256, 256 * sizeof(float), s>>>(net->gpred, 1, 0, 1, V0, nullptr, net->cpart);
     k_sum_parts<<<1, 256, 0, s>>>(net->cpart, kColsumBlocks, 1, net->g + hd.off_b, accumulate);
-    k_head_bwd<<<blocks_for(V0 * c0), 256, 0, s>>>(net->gpred, net->db[0], c0, net->w + hd.off_w, net->gA, V0);
+    k_head_bwd<<<blocks_for(V0 * c0 / 8), 256, 0, s>>>(net->gpred, net->db[0], c0, net->w + hd.off_w, net->gA, V0);
     UCK(cudaGetLastError());
   }
   // decoder levels 0 .. L-2 (the reverse of their forward order); gA holds the gradient of the
