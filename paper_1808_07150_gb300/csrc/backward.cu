@@ -88,9 +88,10 @@ __global__ void __launch_bounds__(1024) k_bwd_table_scan(const unsigned short* c
   if (threadIdx.x == 0) totals[v] = (unsigned)total;
 }
 
-// one batch of at most 128 components, three taps (the item's packing), view subsets
+// one batch of at most 128 components, three taps (the item's packing), view subsets; flat geometries
+// compute their few bins
 bool backward_table_possible(const DevGeom& g) {
-  return !g.bins && g.taps <= 3 && g.bw_nb == 1 && g.n_comp <= 128;
+  return !g.bins && !flat_geometry(g) && g.taps <= 3 && g.bw_nb == 1 && g.n_comp <= 128;
 }
 
 size_t backward_table_recs(const DevGeom& g) {
@@ -127,6 +128,7 @@ cudaError_t backward_table_fill(const DevGeom& g, const unsigned* starts, const 
 
 cudaError_t launch_backward(const DevGeom& g, int subset, int mode, const BwdArgs& a, cudaStream_t s) {
   if (a.items && !backward_table_possible(g)) return cudaErrorInvalidValue;
+  if (flat_geometry(g)) return launch_backward_flat(g, subset, mode, a, s);
   switch (g.taps) {
     case 1: return launch_backward_nt<1>(g, subset, mode, a, s);
     case 2: return launch_backward_nt<2>(g, subset, mode, a, s);

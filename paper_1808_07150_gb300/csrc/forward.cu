@@ -32,6 +32,7 @@ void forward_layout(DevGeom& g, const SegDev* seg, std::vector<int4>& tasks) {
 }
 
 int forward_split(const DevGeom& g, int subset) {
+  if (flat_geometry(g)) return 1;
   if (g.tune[SPDHG_TUNE_FWD_SPLIT]) return g.tune[SPDHG_TUNE_FWD_SPLIT];
   // enough blocks for every SM: one LOR line per block is too few for small subsets
   const int lines = subset_views(g, subset) * g.R * forward_parts(g);
@@ -63,6 +64,7 @@ int forward_entry_groups(const DevGeom& g) {
 }
 
 cudaError_t launch_forward(const DevGeom& g, int subset, int mode, const FwdArgs& a, cudaStream_t s) {
+  if (flat_geometry(g)) return launch_forward_flat(g, subset, mode, a, s);
   switch (g.taps) {
     case 1: return launch_forward_nt<1>(g, subset, mode, a, s);
     case 2: return launch_forward_nt<2>(g, subset, mode, a, s);

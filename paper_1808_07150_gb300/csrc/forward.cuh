@@ -121,6 +121,44 @@ __device__ __forceinline__ void cp_async4_if(unsigned d, const float* s, bool on
                : "memory");
 }
 
+// What a mode does with one bin's line integral `sum` (plane p of line (v, r); l: the view's place in
+// the subset).
+template <int MODE>
+__device__ __forceinline__ void forward_epilogue(const DevGeom& g, const FwdArgs& a, int subset, int v, int l, int r, int p, float sum) {
+  const size_t j = ((size_t)v * g.R + r) * g.P + p;
+  const size_t jl = ((size_t)l * g.R + r) * g.P + p;  // subset-local index (= j for bin subsets)
+  if (!bin_in_subset(g, subset, j)) {  // a bin of another subset: not written; no dual change
+    if (MODE == FWD_DATA || MODE == FWD_EM) a.wdy[jl] = 0.f;
+    return;
+  }
+  const float mu = a.mult ? a.mult[j] : 1.f;
+  if (MODE == FWD_EM) {
+    // EM ratio backprojected by P^T = L^T diag(mult): mult_j b_j / ((P x)_j + r_j)  (Eq. EQU:OSEM)
+    const float bj = a.b[j];
+    a.wdy[jl] = bj > 0.f ? mu * bj / fmaf(mu, sum, a.r[j]) : 0.f;
+  } else if (MODE == FWD_PROJECT) {
+    a.out[j] = mu * sum;
+  } else if (MODE == FWD_SIGMA) {
+    // sigma_j = gamma rho / (P_i 1)_j,  (P_i 1)_j = mult_j * chord_j  (Eq. EQU:STEPSIZE:PRECOND)
+    const float a1 = mu * sum;
+    a.out[j] = a1 > 0.f ? a.gamma_rho / a1 : 0.f;
+  } else {
+    // KL dual prox on this bin:  y+ = prox_{sigma varphi*}(y + sigma (P_i x)_j), evaluated as
+    // 2 (u - sigma b) / (u + 1 + sqrt((u - 1)^2 + 4 sigma b)),  u = y + sigma ((P_i x)_j + r_j),
+    // which equals 1/2 [u + 1 - sqrt((u - 1)^2 + 4 sigma b)] without its cancellation.
+    const float sigma = a.sigma[j];
+    const float yj = a.y[j];
+    const float bj = a.b[j];
+    const float u = fmaf(sigma, fmaf(mu, sum, a.r[j]), yj);
+    const float sb = sigma * bj;
+    const float um = u - 1.f;
+    const float root = sqrtf(fmaf(um, um, 4.f * sb));
+    const float yn = 2.f * (u - sb) / (u + 1.f + root);
+    a.y[j] = yn;
+    a.wdy[jl] = mu * (yn - yj);
+  }
+}
+
 // Forward projection.  Block (line, row part, plane part) owns the rows [row_lo, row_hi) of one
 // transaxial LOR line (view, radial bin) and a contiguous range of the geometry's plane tasks (up to
 // four words of 32 consecutive planes of one segment); a warp owns one task, lane l plane q0 + l of
@@ -350,40 +388,7 @@ __global__ void __launch_bounds__(kFwdMaxWarps * 32, GROUPS ? 3 : 2)
 #pragma unroll
   for (int w = 0; w < 4; ++w) {
     if (!(writes && w < words && q + 32 * w < sd.n)) continue;
-    const float sum = acc[w];
-    const int p = sd.p0 + q + 32 * w;
-    const size_t j = ((size_t)v * g.R + r) * g.P + p;
-    const size_t jl = ((size_t)l * g.R + r) * g.P + p;  // subset-local index (= j for bin subsets)
-    if (!bin_in_subset(g, subset, j)) {  // a bin of another subset: not written; no dual change
-      if (MODE == FWD_DATA || MODE == FWD_EM) a.wdy[jl] = 0.f;
-      continue;
-    }
-    const float mu = a.mult ? a.mult[j] : 1.f;
-    if (MODE == FWD_EM) {
-      // EM ratio backprojected by P^T = L^T diag(mult): mult_j b_j / ((P x)_j + r_j)  (Eq. EQU:OSEM)
-      const float bj = a.b[j];
-      a.wdy[jl] = bj > 0.f ? mu * bj / fmaf(mu, sum, a.r[j]) : 0.f;
-    } else if (MODE == FWD_PROJECT) {
-      a.out[j] = mu * sum;
-    } else if (MODE == FWD_SIGMA) {
-      // sigma_j = gamma rho / (P_i 1)_j,  (P_i 1)_j = mult_j * chord_j  (Eq. EQU:STEPSIZE:PRECOND)
-      const float a1 = mu * sum;
-      a.out[j] = a1 > 0.f ? a.gamma_rho / a1 : 0.f;
-    } else {
-      // KL dual prox on this bin:  y+ = prox_{sigma varphi*}(y + sigma (P_i x)_j), evaluated as
-      // 2 (u - sigma b) / (u + 1 + sqrt((u - 1)^2 + 4 sigma b)),  u = y + sigma ((P_i x)_j + r_j),
-      // which equals 1/2 [u + 1 - sqrt((u - 1)^2 + 4 sigma b)] without its cancellation.
-      const float sigma = a.sigma[j];
-      const float yj = a.y[j];
-      const float bj = a.b[j];
-      const float u = fmaf(sigma, fmaf(mu, sum, a.r[j]), yj);
-      const float sb = sigma * bj;
-      const float um = u - 1.f;
-      const float root = sqrtf(fmaf(um, um, 4.f * sb));
-      const float yn = 2.f * (u - sb) / (u + 1.f + root);
-      a.y[j] = yn;
-      a.wdy[jl] = mu * (yn - yj);
-    }
+    forward_epilogue<MODE>(g, a, subset, v, l, r, sd.p0 + q + 32 * w, acc[w]);
   }
 }
 

@@ -169,6 +169,10 @@ size_t backward_table_recs(const DevGeom& g);
 // tile, staged rows and component batches of a geometry (host tables; see backward.cu)
 void backward_layout(DevGeom& g, const SegDev* seg, CompDev* comp, std::vector<int2>& slots, std::vector<BwdBatch>& batches);
 
+// one slice and one untilted plane per line: the kernels of flat.cu serve it
+bool flat_geometry(const DevGeom& g);
+cudaError_t launch_forward_flat(const DevGeom& g, int subset, int mode, const FwdArgs& a, cudaStream_t s);
+cudaError_t launch_backward_flat(const DevGeom& g, int subset, int mode, const BwdArgs& a, cudaStream_t s);
 cudaError_t launch_forward(const DevGeom& g, int subset, int mode, const FwdArgs& a, cudaStream_t s);
 cudaError_t launch_backward(const DevGeom& g, int subset, int mode, const BwdArgs& a, cudaStream_t s);
 // w_local = y * mult over the bins of subset i (y or mult null: ones); for bin subsets the
