@@ -19,7 +19,32 @@ void backward_layout(DevGeom& g, const SegDev* seg, CompDev* comp, std::vector<i
     const double diag = sqrt(4.0 * cpw * cpw + 16.0);
     return (int)floor(diag * inv * (1.0 + 1e-5) + 4.0 * kBinMargin) + 1;
   };
-  auto run = [&](int c) { return comp[c].qhi - comp[c].qlo + pad; };  // its planes and one frame
+  // Runs of staged planes.  A component whose bins hold every plane of its range has its own run,
+  // followed by a frame of taps - 1 zeros.  One that holds every second plane is staged without the
+  // gaps; the lane masks keep its gather inside it, so the components of a segment share one run per
+  // parity and no frame.  344 x 344 x 127 voxels, 121 components over 837 planes: 8200 slots with runs
+  // and gaps per component, 837 shared.
+  struct Run { int seg, lo, hi, slot; };
+  g.bw_step2 = 0;
+  std::vector<int> run_of(g.n_comp);
+  std::vector<Run> runs;
+  for (int c = 0; c < g.n_comp; ++c) {
+    const int step = 1 + comp[c].smask;
+    const int hi = comp[c].qlo + (comp[c].qhi - comp[c].qlo - 1) / step * step + 1;
+    comp[c].len = hi - comp[c].qlo + (step == 2 ? 1 : pad);
+    g.bw_step2 |= comp[c].smask;
+    int k = (int)runs.size();
+    if (step == 2) {
+      for (k = 0; k < (int)runs.size(); ++k)
+        if (runs[k].seg == comp[c].seg && ((runs[k].lo ^ comp[c].qlo) & 1) == 0) break;
+    }
+    if (k == (int)runs.size()) runs.push_back(Run{comp[c].seg, comp[c].qlo, hi, -1});
+    runs[k].lo = std::min(runs[k].lo, comp[c].qlo);
+    runs[k].hi = std::max(runs[k].hi, hi);
+    run_of[c] = k;
+  }
+  auto frame = [&](int c) { return comp[c].smask ? 0 : pad; };
+  auto run = [&](int c) { return (runs[run_of[c]].hi - runs[run_of[c]].lo + comp[c].smask) / (1 + comp[c].smask) + frame(c); };
   int widest = 0;
   for (int c = 0; c < g.n_comp; ++c) widest = std::max(widest, run(c) + pad);
   // four columns per warp share a block's set-up and a warp's item records (171 x 171: 98 us against
@@ -39,14 +64,18 @@ void backward_layout(DevGeom& g, const SegDev* seg, CompDev* comp, std::vector<i
     BwdBatch b{c, c, (int)slots.size(), 0, 0, pad};
     std::vector<int2> zeros;
     for (int k = 0; k < pad; ++k) zeros.push_back(make_int2(k, -1));
-    while (c < g.n_comp && (c == b.c0 || b.slots + run(c) <= room)) {
-      comp[c].slot = b.slots - pad;
-      comp[c].len = comp[c].qhi - comp[c].qlo + pad;
-      for (int q = comp[c].qlo; q < comp[c].qhi; ++q, ++b.slots) {
-        if (((q - comp[c].qlo) & comp[c].smask) == 0) slots.push_back(make_int2(b.slots, seg[comp[c].seg].p0 + q));
-        else zeros.push_back(make_int2(b.slots, -1));
+    for (Run& q : runs) q.slot = -1;
+    while (c < g.n_comp) {
+      Run& q = runs[run_of[c]];
+      const int step = 1 + comp[c].smask;
+      if (q.slot < 0) {
+        if (c > b.c0 && b.slots + run(c) > room) break;
+        q.slot = b.slots;
+        for (int p = q.lo; p < q.hi; p += step) slots.push_back(make_int2(b.slots++, seg[q.seg].p0 + p));
+        for (int k = 0; k < frame(c); ++k) zeros.push_back(make_int2(b.slots++, -1));
       }
-      for (int k = 0; k < pad; ++k) zeros.push_back(make_int2(b.slots++, -1));
+      // a step-2 record counts from the component's first plane, the others from the frame below it
+      comp[c].slot = step == 2 ? q.slot + (comp[c].qlo - q.lo) / 2 : q.slot - pad;
       ++c;
     }
     b.c1 = c;

@@ -83,11 +83,19 @@ __device__ __forceinline__ unsigned lane_range(int off, int len) {
 }
 
 // Item record word: 4 x (staged offset + kOffBias) | (taps - 1); the bias keeps it non-negative.
+// The words of step-2 components are marked kStep2; their low bits are a parity and kMoreTaps.
 constexpr int kOffBias = 256;
+constexpr unsigned kStep2 = 1u << 31, kMoreTaps = 2u;
 
-// One tap of ZK slices: acc[k] += L * shared[addr + 128 k + OFF] in the lanes that m[k] holds.  The
+// lane masks per record: one set, and one for the taps above the second of a step-2 component
+template <int NT, bool MASHED>
+__host__ __device__ constexpr int mask_sets() {
+  return MASHED && NT > 2 ? 2 : 1;
+}
+
+// One tap of ZK slices: acc[k] += L * shared[addr + STRIDE k + OFF] in the lanes that m[k] holds.  The
 // predicates are explicit because the compiler turns the equivalent branches into jumps.
-template <int ZK, int OFF>
+template <int ZK, int OFF, int STRIDE = 128>
 __device__ __forceinline__ void tap_fma(unsigned addr, float L, const unsigned* m, unsigned bit, float* acc) {
 #pragma unroll
   for (int k = 0; k < ZK; ++k)
@@ -98,29 +106,57 @@ __device__ __forceinline__ void tap_fma(unsigned addr, float L, const unsigned* 
         "@p ld.shared.f32 f, [%3];\n\t"
         "@p fma.rn.f32 %0, %4, f, %0;\n\t}\n"
         : "+f"(acc[k])
-        : "r"(m[k]), "r"(bit), "r"(addr + (OFF + 128 * k)), "f"(L));
+        : "r"(m[k]), "r"(bit), "r"(addr + (OFF + STRIDE * k)), "f"(L));
 }
 
 // Accumulates one column's item records [i0, i1): voxel lane + 32 k adds sum_t L_t buf[off + lane +
 // 32 k + t] where bit `lane` of the item's mask k is set.  `base` is the shared address of the
-// buffer's slot lane - kOffBias.
-template <int NT, int ZK>
+// buffer's slot lane - kOffBias.  A step-2 component holds planes of one parity, staged without
+// gaps, so every second one of a lane's taps meets a plane: with u = lane + parity the lane reads slot
+// u >> 1 in place of lane, at tap 0 where u is odd and tap 1 where it is even, and if the item has more
+// than two taps also the slot after it, with masks of its own, at tap 2 or 3.  A tap of no weight
+// reads nothing, so that no plane outside the LOR's slices is touched.
+template <int NT, int ZK, bool MASHED>
 __device__ __forceinline__ void gather_items(unsigned base, const float4* recA, const uint4* recM, const int* recO,
                                              int i0, int i1, unsigned bit, float* acc) {
-  constexpr int MQ = (ZK + 3) / 4;
+  constexpr int MQ = (ZK + 3) / 4, MR = MQ * mask_sets<NT, MASHED>();
 #pragma unroll 1
   for (int it = i0; it < i1; ++it) {
     const float4 A = recA[it];
     const unsigned word = NT > 3 ? (unsigned)recO[it] : __float_as_uint(A.w);
-    const unsigned addr = base + (word & ~3u);
+    const unsigned addr = base + (word & ~(kStep2 | 3u));
     unsigned m[4 * MQ];
 #pragma unroll
     for (int q = 0; q < MQ; ++q) {
-      const uint4 u = recM[it * MQ + q];
+      const uint4 u = recM[it * MR + q];
       m[4 * q] = u.x;
       m[4 * q + 1] = u.y;
       m[4 * q + 2] = u.z;
       m[4 * q + 3] = u.w;
+    }
+    if constexpr (MASHED) {
+      if (word & kStep2) {
+        const int lane = threadIdx.x & 31, u = lane + (int)(word & 1u);
+        const unsigned half = addr + 4 * ((u >> 1) - lane);
+        const bool odd = u & 1;
+        const float L = odd ? A.x : A.y;
+        tap_fma<ZK, 0, 64>(half, L, m, L != 0.f ? bit : 0u, acc);
+        if constexpr (NT > 2) {
+          if (word & kMoreTaps) {
+#pragma unroll
+            for (int q = 0; q < MQ; ++q) {
+              const uint4 v = recM[it * MR + MQ + q];
+              m[4 * q] = v.x;
+              m[4 * q + 1] = v.y;
+              m[4 * q + 2] = v.z;
+              m[4 * q + 3] = v.w;
+            }
+            const float L2 = odd ? A.z : (NT > 3 ? A.w : 0.f);
+            tap_fma<ZK, 4, 64>(half, L2, m, L2 != 0.f ? bit : 0u, acc);
+          }
+        }
+        continue;
+      }
     }
     tap_fma<ZK, 0>(addr, A.x, m, bit, acc);
     if constexpr (NT > 1) {
@@ -149,9 +185,7 @@ __device__ __forceinline__ float ld_now(const float* p) {
 // Backprojection.  A block of 8 warps owns a tile of 2 CPW x 4 voxel columns, warp w the CPW
 // columns at (w & 1, w >> 1).  Work is cut into stages (view group, component batch): the radial
 // rows of the group's views that the tile's footprints touch are copied into shared memory
-// (cp.async), every LOR component as its own run of planes framed by NT - 1 zeros, with zeros also
-// where a plane does not include the component, so that mashed and plain geometries share one
-// gather.  The (bin, interval, component) items of a warp's columns are read from the table
+// (cp.async) as runs of planes (backward_layout), those of plain segments framed by NT - 1 zeros.  The (bin, interval, component) items of a warp's columns are read from the table
 // spdhg_setup builds (TAB) or computed, one item per lane, and expanded to records in shared memory;
 // a column's records are then accumulated with lanes along z, 32 slices per register.  A record
 // carries, per 32 slices, the mask of the lanes whose planes lie in the run: one AND decides a lane,
@@ -166,21 +200,22 @@ __device__ __forceinline__ float ld_now(const float* p) {
 // view of 344 x 837 bins, BWD_UPDATE 137 -> 97 us (302 MB algorithmic, 3.1 TB/s) against a block of
 // 16 one-column warps whose epilogues ran in step; 171 x 171 x 92, 12-13 views x 250 planes,
 // 128 -> 94 us; 128 x 128 x 64, 8-9 views, three mashed components, 51 -> 35 us; 64 x 64 x 1, 9 views,
-// 19 -> 12 us.  Two buffers per block (the next stage's copies in flight) gave nothing over one:
+// 19 -> 12 us; 344 x 344 x 127, one view, 121 components over 837 planes (BWD_OUT) 767 -> 747 us
+// (870 when every component had its own gapped run).  Two buffers per block (the next stage's copies in flight) gave nothing over one:
 // the other blocks of the SM cover the wait.  Frames of 31 zeros instead of lane masks (8-byte
 // records, no masks) took the same time and room for fewer views.  Five blocks per SM spill.
-template <int NT, int ZK, int CPW, bool SINGLE, bool TAB>
+template <int NT, int ZK, int CPW, bool SINGLE, bool TAB, bool MASHED>
 __global__ void __launch_bounds__(kBwdWarps * 32, ZK <= 4 ? 4 : 3)
     k_backward(const __grid_constant__ DevGeom g, int subset, int groups, int mode, const __grid_constant__ BwdArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
   constexpr int PAD = NT - 1;
-  constexpr int MQ = (ZK + 3) / 4;
+  constexpr int MQ = (ZK + 3) / 4, MR = MQ * mask_sets<NT, MASHED>();
   constexpr int TX = 2 * CPW, TY = 4;
   const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
   const unsigned bit = 1u << lane;
   float4* recA = reinterpret_cast<float4*>(smem) + wi * kBwdFill;
-  uint4* recM = reinterpret_cast<uint4*>(smem + kBwdWarps * kBwdFill * 16) + wi * kBwdFill * MQ;
-  unsigned char* rest = smem + kBwdWarps * kBwdFill * 16 * (1 + MQ);
+  uint4* recM = reinterpret_cast<uint4*>(smem + kBwdWarps * kBwdFill * 16) + wi * kBwdFill * MR;
+  unsigned char* rest = smem + kBwdWarps * kBwdFill * 16 * (1 + MR);
   int* recO = reinterpret_cast<int*>(rest) + wi * kBwdFill;
   if (NT > 3) rest += kBwdWarps * kBwdFill * 4;
   const int pix_cap = CPW * g.bw_views * g.bw_cand;
@@ -218,7 +253,7 @@ __global__ void __launch_bounds__(kBwdWarps * 32, ZK <= 4 ? 4 : 3)
       dst += g.bw_rows * bt.slots;
     }
   };
-  // zeros of batch b: frames and planes that miss a component; the copies never touch them
+  // zeros of batch b: the frames; the copies never touch them
   auto zeros = [&](int b) {
     const BwdBatch bt = g.bw_batch[b];
     for (int p = threadIdx.x; p < bt.zeros; p += kBwdWarps * 32) {
@@ -299,7 +334,7 @@ __global__ void __launch_bounds__(kBwdWarps * 32, ZK <= 4 ? 4 : 3)
       __syncwarp();
       if (i < total) {
         float L[4] = {0.f, 0.f, 0.f, 0.f};
-        int row_slot, jp, len;
+        int row_slot, jp, len, smask;
         if (TAB) {
           const unsigned pk = __float_as_uint(pre.w);
           L[0] = pre.x;
@@ -308,6 +343,7 @@ __global__ void __launch_bounds__(kBwdWarps * 32, ZK <= 4 ? 4 : 3)
           row_slot = (int)(pk & 0xFFFFu);
           jp = (int)((pk >> 16) & 0x1FFu) - 256;
           len = g.comp[pk >> 25].len;
+          smask = MASHED ? g.comp[pk >> 25].smask : 0;
         } else {
           const int pi = i / cc, ci = cb + (i - pi * cc);
           const PixItem Q = pix[pi];
@@ -316,22 +352,34 @@ __global__ void __launch_bounds__(kBwdWarps * 32, ZK <= 4 ? 4 : 3)
           row_slot = Q.row * slots + cd.slot;
           jp = j0 - cd.qlo + PAD;
           len = cd.len;
+          smask = MASHED ? cd.smask : 0;
         }
         int nt = 1;
 #pragma unroll
         for (int k = 1; k < NT; ++k)
           if (L[k] != 0.f) nt = k + 1;
-        const int word = 4 * (row_slot + jp + kOffBias) | (nt - 1);
+        int word = 4 * (row_slot + jp + kOffBias) | (nt - 1);
+        const bool step2 = MASHED && smask;
+        if (step2) {
+          jp -= PAD - 1;  // tap 1 of lane b meets plane b + jp of the component, if that is even
+          word = (4 * (row_slot + (jp >> 1) + kOffBias) | (jp & 1)) | (nt > 2 ? (int)kMoreTaps : 0) | (int)kStep2;
+        }
         recA[lane] = make_float4(L[0], L[1], L[2], NT > 3 ? L[3] : __int_as_float(word));
         if (NT > 3) recO[lane] = word;
+        auto masks = [&](uint4* to, int off) {
 #pragma unroll
-        for (int q = 0; q < MQ; ++q) {
-          uint4 m;
-          m.x = lane_range(jp + 128 * q, len);
-          m.y = ZK > 1 ? lane_range(jp + 128 * q + 32, len) : 0u;
-          m.z = ZK > 2 ? lane_range(jp + 128 * q + 64, len) : 0u;
-          m.w = ZK > 3 ? lane_range(jp + 128 * q + 96, len) : 0u;
-          recM[lane * MQ + q] = m;
+          for (int q = 0; q < MQ; ++q) {
+            uint4 m;
+            m.x = lane_range(off + 128 * q, len);
+            m.y = ZK > 1 ? lane_range(off + 128 * q + 32, len) : 0u;
+            m.z = ZK > 2 ? lane_range(off + 128 * q + 64, len) : 0u;
+            m.w = ZK > 3 ? lane_range(off + 128 * q + 96, len) : 0u;
+            to[q] = m;
+          }
+        };
+        masks(recM + lane * MR, jp);
+        if constexpr (mask_sets<NT, MASHED>() > 1) {
+          if (step2 && nt > 2) masks(recM + lane * MR + MQ, jp + 2);
         }
       }
       base = it;
@@ -369,7 +417,7 @@ __global__ void __launch_bounds__(kBwdWarps * 32, ZK <= 4 ? 4 : 3)
       while (it < end) {
         if (it == filled) fill();
         const int e = min(end, filled);
-        gather_items<NT, ZK>(buf, recA, recM, recO, it - base, e - base, bit, ac);
+        gather_items<NT, ZK, MASHED>(buf, recA, recM, recO, it - base, e - base, bit, ac);
         it = e;
       }
       if (!last) {
@@ -472,37 +520,38 @@ inline int bwd_groups(const DevGeom& g, int subset) {
   return (most + g.bw_views - 1) / g.bw_views;
 }
 
-template <int NT, int ZK, int CPW, bool SINGLE, bool TAB>
+template <int NT, int ZK, int CPW, bool SINGLE, bool TAB, bool MASHED>
 cudaError_t bwd_run(const DevGeom& g, int subset, int mode, const BwdArgs& a, cudaStream_t s) {
   const int groups = bwd_groups(g, subset);
-  size_t smem = (size_t)kBwdWarps * kBwdFill * 16 * (1 + (ZK + 3) / 4);
+  size_t smem = (size_t)kBwdWarps * kBwdFill * 16 * (1 + (ZK + 3) / 4 * mask_sets<NT, MASHED>());
   if (NT > 3) smem += (size_t)kBwdWarps * kBwdFill * 4;
   if (!TAB) smem += ((size_t)kBwdWarps * CPW * g.bw_views * g.bw_cand * sizeof(PixItem) + 15) & ~(size_t)15;
   if (!SINGLE) smem += (size_t)kBwdWarps * CPW * ZK * 128;
   smem += (size_t)g.bw_buf * sizeof(float);
   if (smem > 220 * 1024) return cudaErrorInvalidValue;
-  auto kern = k_backward<NT, ZK, CPW, SINGLE, TAB>;
+  auto kern = k_backward<NT, ZK, CPW, SINGLE, TAB, MASHED>;
   cudaError_t e = allow_dynamic_smem(kern, smem);
   if (e != cudaSuccess) return e;
   kern<<<bwd_tiles(g), kBwdWarps * 32, smem, s>>>(g, subset, groups, mode, a);
   return cudaGetLastError();
 }
 
-template <int NT, int ZK, bool TAB>
+template <int NT, int ZK, bool TAB, bool MASHED>
 cudaError_t bwd_shape(const DevGeom& g, int subset, int mode, const BwdArgs& a, cudaStream_t s) {
-  if (g.bw_cpw == 1) return bwd_run<NT, ZK, 1, false, TAB>(g, subset, mode, a, s);
-  if (bwd_groups(g, subset) * g.bw_nb == 1) return bwd_run<NT, ZK, 4, true, TAB>(g, subset, mode, a, s);
-  return bwd_run<NT, ZK, 4, false, TAB>(g, subset, mode, a, s);
+  if (g.bw_cpw == 1) return bwd_run<NT, ZK, 1, false, TAB, MASHED>(g, subset, mode, a, s);
+  if (bwd_groups(g, subset) * g.bw_nb == 1) return bwd_run<NT, ZK, 4, true, TAB, MASHED>(g, subset, mode, a, s);
+  return bwd_run<NT, ZK, 4, false, TAB, MASHED>(g, subset, mode, a, s);
 }
 
 template <int NT, int ZK>
 cudaError_t bwd_tab(const DevGeom& g, int subset, int mode, const BwdArgs& a, cudaStream_t s) {
   if constexpr (NT <= 3) {
-    if (a.items) return bwd_shape<NT, ZK, true>(g, subset, mode, a, s);
+    if (a.items)
+      return g.bw_step2 ? bwd_shape<NT, ZK, true, true>(g, subset, mode, a, s) : bwd_shape<NT, ZK, true, false>(g, subset, mode, a, s);
   } else {
     if (a.items) return cudaErrorInvalidValue;
   }
-  return bwd_shape<NT, ZK, false>(g, subset, mode, a, s);
+  return g.bw_step2 ? bwd_shape<NT, ZK, false, true>(g, subset, mode, a, s) : bwd_shape<NT, ZK, false, false>(g, subset, mode, a, s);
 }
 
 // instantiated per tap count in backward_taps<NT>.cu

@@ -32,7 +32,7 @@ struct CompDev {
   int seg;
   int qlo, qhi, smask;
   int jlo, jhi;  // range of the tap offset j0 of any pixel of any LOR of the component (host bound)
-  int slot, len; // backprojector: staged slot taps - 1 below the component's first plane, its planes + taps - 1
+  int slot, len; // backprojector: staged slot of its first plane (step 1: taps - 1 below it); lanes that meet it
 };
 
 // Components [c0, c1) whose planes the backprojector stages together: rows of `slots` floats; entries
@@ -64,6 +64,7 @@ struct DevGeom {
   // bins per column and view, component batches, most views per stage, floats of the staging buffer; the batches, and their
   // copies (slot, plane) and zero slots
   int bw_cpw, bw_rows, bw_cand, bw_nb, bw_views, bw_buf;
+  int bw_step2;          // 1: some component has step 2
   const BwdBatch* bw_batch;
   const int2* bw_slots;
   int n_tasks;           // plane tasks of the forward projector, segment-major
