@@ -24,7 +24,7 @@ void backward_layout(DevGeom& g, const SegDev* seg, CompDev* comp, std::vector<i
   // gaps; the lane masks keep its gather inside it, so the components of a segment share one run per
   // parity and no frame.  344 x 344 x 127 voxels, 121 components over 837 planes: 8200 slots with runs
   // and gaps per component, 837 shared.
-  struct Run { int seg, lo, hi, slot; };
+  struct Run { int seg, step, lo, hi, slot; };
   g.bw_step2 = 0;
   std::vector<int> run_of(g.n_comp);
   std::vector<Run> runs;
@@ -36,17 +36,20 @@ void backward_layout(DevGeom& g, const SegDev* seg, CompDev* comp, std::vector<i
     int k = (int)runs.size();
     if (step == 2) {
       for (k = 0; k < (int)runs.size(); ++k)
-        if (runs[k].seg == comp[c].seg && ((runs[k].lo ^ comp[c].qlo) & 1) == 0) break;
+        if (runs[k].step == 2 && runs[k].seg == comp[c].seg && ((runs[k].lo ^ comp[c].qlo) & 1) == 0) break;
     }
-    if (k == (int)runs.size()) runs.push_back(Run{comp[c].seg, comp[c].qlo, hi, -1});
+    if (k == (int)runs.size()) runs.push_back(Run{comp[c].seg, step, comp[c].qlo, hi, -1});
     runs[k].lo = std::min(runs[k].lo, comp[c].qlo);
     runs[k].hi = std::max(runs[k].hi, hi);
     run_of[c] = k;
   }
-  auto frame = [&](int c) { return comp[c].smask ? 0 : pad; };
-  auto run = [&](int c) { return (runs[run_of[c]].hi - runs[run_of[c]].lo + comp[c].smask) / (1 + comp[c].smask) + frame(c); };
+  // slots a component's run takes at most (a plain run may need a frame on either side)
+  auto run = [&](int c) {
+    const Run& q = runs[run_of[c]];
+    return (q.hi - q.lo + q.step - 1) / q.step + (q.step == 1 ? 2 * pad : 0);
+  };
   int widest = 0;
-  for (int c = 0; c < g.n_comp; ++c) widest = std::max(widest, run(c) + pad);
+  for (int c = 0; c < g.n_comp; ++c) widest = std::max(widest, run(c));
   // four columns per warp share a block's set-up and a warp's item records (171 x 171: 98 us against
   // 149 with one column, 128 x 128: 35 against 40); one column per warp where four would leave fewer
   // than two blocks per SM, or rows too long for shared memory
@@ -63,19 +66,26 @@ void backward_layout(DevGeom& g, const SegDev* seg, CompDev* comp, std::vector<i
   for (int c = 0; c < g.n_comp;) {
     BwdBatch b{c, c, (int)slots.size(), 0, 0, pad};
     std::vector<int2> zeros;
-    for (int k = 0; k < pad; ++k) zeros.push_back(make_int2(k, -1));
+    bool framed = true;  // the slots before the next run are a frame
+    auto frame = [&]() {
+      for (int k = 0; k < pad; ++k) zeros.push_back(make_int2(b.slots++, -1));
+      framed = true;
+    };
+    b.slots = 0;
+    frame();
     for (Run& q : runs) q.slot = -1;
     while (c < g.n_comp) {
       Run& q = runs[run_of[c]];
-      const int step = 1 + comp[c].smask;
       if (q.slot < 0) {
-        if (c > b.c0 && b.slots + run(c) > room) break;
+        if (c > b.c0 && b.slots + run(c) - (q.step == 1 && framed ? pad : 0) > room) break;
+        if (q.step == 1 && !framed) frame();
         q.slot = b.slots;
-        for (int p = q.lo; p < q.hi; p += step) slots.push_back(make_int2(b.slots++, seg[q.seg].p0 + p));
-        for (int k = 0; k < frame(c); ++k) zeros.push_back(make_int2(b.slots++, -1));
+        for (int p = q.lo; p < q.hi; p += q.step) slots.push_back(make_int2(b.slots++, seg[q.seg].p0 + p));
+        if (q.step == 1) frame();
+        else framed = false;
       }
       // a step-2 record counts from the component's first plane, the others from the frame below it
-      comp[c].slot = step == 2 ? q.slot + (comp[c].qlo - q.lo) / 2 : q.slot - pad;
+      comp[c].slot = q.step == 2 ? q.slot + (comp[c].qlo - q.lo) / 2 : q.slot - pad;
       ++c;
     }
     b.c1 = c;
