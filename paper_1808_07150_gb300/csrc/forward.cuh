@@ -173,7 +173,7 @@ __device__ __forceinline__ void forward_epilogue(const DevGeom& g, const FwdArgs
 // of every chunk; group 0 adds the other groups' sums in group order.  When several row parts share
 // a line, each writes partial plane sums and the last one to finish reduces them in a fixed order.
 //
-// Bound: instruction issue (62 % active at the mMR scale, 44 M warp instructions, 67 M before with two
+// Bound: instruction issue (60 % active at the mMR scale, 36 M warp instructions, 58 M before with two
 // words per warp), then latency with 344 lines on 152 SMs.  So a record's reads and address serve up
 // to four words, and the copies of aligned columns are dealt out in 16-byte pieces.  Measured on
 // GB300, per launch: 344 x 344 x 127 voxels, one view of 344 x 837 bins, 92 -> 63 us; 171 x 171 x 92,
