@@ -1,5 +1,5 @@
-// 3x3x3 convolutions of the learned warm start (forward, data gradient, weight gradient) on the tensor
-// cores (tcgen05, BF16 x BF16 -> FP32 in TMEM) without an im2col gather.
+// 3x3x3 convolutions of the learned warm start (forward, data gradient) on the tensor cores (tcgen05,
+// BF16 x BF16 -> FP32 in TMEM) without an im2col gather.
 //
 // A tile is 16 consecutive x positions x 8 consecutive z slices at one y: 128 voxels, row r = 8 m + j
 // <-> voxel (y, x0 + m, z0 + j).  Its input halo (3 y x 18 x x 10 z voxels, zero outside the volume) is
@@ -12,10 +12,9 @@
 // channels, where the step's products take 4), then the halo copies; so blocks are persistent, three
 // halos are in flight, and the accumulator of one tile is read while the next tile's MMAs run.  Measured
 // on GB300, 128 x 128 x 64 voxels: 32 -> 16 channels 202 -> 146 us, 16 -> 16 104 -> 58 us, 8 -> 16 101 -> 45 us
-// (from the gather); 64 -> 32 at 64 x 64 x 32 165 -> 70 us, 128 -> 128 at 16 x 16 x 8 88 -> 23 us (gather);
-// weight gradients 32 -> 16 658 -> 186 us, 16 -> 16 308 -> 108 us, 128 -> 64 174 -> 62 us (gather).  Inference
-// 1411 -> 804 us, gradients of a mini-batch of four 21.98 -> 11.91 ms.  128 threads: 897 us and 13.8 ms;
-// 512: 884 us and 12.8 ms.
+// (from the gather); 64 -> 32 at 64 x 64 x 32 165 -> 70 us, 128 -> 128 at 16 x 16 x 8 88 -> 23 us (gather).
+// Inference 1411 -> 803 us, gradients of a mini-batch of four 22.0 -> 16.8 ms.  Inference with 128 threads:
+// 897 us; with 512: 884 us.
 // Included by igemm.cu, whose error flag and mode table it shares.
 #pragma once
 
@@ -307,170 +306,6 @@ cudaError_t launch_conv3(const GemmArgs& g, cudaStream_t s) {
   const dim3 grid(tiles, g.N / Nt);
   if (C == 64) return go(k_conv3_deep<64>, grid, smem, Nt);
   return go(k_conv3_deep<128>, grid, smem, Nt);
-}
-
-// ------------------------------------------------------------------------------------------
-// weight gradient: D[(tap, ci)][co] = sum over voxels v of in[v + tap][ci] g[v][co]
-//
-// The reduction runs over the tile's voxels, so both operands are MN-major: a core matrix is a z-run
-// of 8 voxels x 8 channels, the same bytes as above.  The halo is laid out by planes (dy, group), all
-// of one size, so the M blocks of one (dx, dz) are the planes in order: rows (dy, ci) of three taps at
-// once, 3 C rows in M = 128 chunks, and a plane of ones after them whose rows sum the columns of g (the
-// bias gradient).  The nine (dx, dz) accumulators stay in TMEM over all tiles of a persistent block; its
-// partial sums are then reduced over the blocks in a fixed order.
-// ------------------------------------------------------------------------------------------
-
-template <int C>
-struct Wg {
-  static constexpr int CG = C / 8, PLANES = 3 * CG;
-  static constexpr int CHUNKS = (3 * C + 127) / 128;           // M = 128 chunks
-  static constexpr bool ONES = 3 * C < CHUNKS * 128;           // a spare plane for the bias gradient
-  static constexpr int BUFS = C <= 32 ? 3 : (C == 64 ? 2 : 1);
-  static constexpr uint32_t GP = HPL * 16;                     // bytes of a plane
-  static constexpr uint32_t ABYTES = (PLANES + (ONES ? 1 : 0)) * GP;
-};
-
-template <int C>
-__global__ void __launch_bounds__(CTHREADS) k_wgrad3(const __grid_constant__ GemmArgs g, int tiles, int Nt, float* bias_part) {
-  using W = Wg<C>;
-  constexpr int CG = W::CG, BUFS = W::BUFS;
-  constexpr uint32_t GP = W::GP;
-  extern __shared__ __align__(1024) unsigned char smem[];
-  __shared__ uint64_t mbar[BUFS];
-  __shared__ uint32_t tmem_slot;
-  const int tid = threadIdx.x, warp = tid >> 5, n_first = blockIdx.y * Nt, NG = Nt >> 3;
-  const uint32_t sh = umma::smem_u32(smem), bbytes = (uint32_t)NG * 2048, buf_bytes = W::ABYTES + bbytes;
-  uint32_t ncols = 32;
-  while ((int)ncols < 9 * Nt * W::CHUNKS) ncols <<= 1;
-  if (warp == 0) umma::tmem_alloc(&tmem_slot, ncols);
-  if (tid == 0) {
-    for (int k = 0; k < BUFS; ++k) umma::mbar_init(&mbar[k], 1);
-    umma::fence_mbar_init();
-  }
-  if (W::ONES) {  // one in the first channel of every voxel
-    for (int i = tid; i < BUFS * HPL; i += CTHREADS) {
-      const int k = i / HPL, h = i - k * HPL;
-      *reinterpret_cast<uint4*>(smem + k * buf_bytes + W::PLANES * GP + h * 16) = make_uint4(0x3F80u, 0u, 0u, 0u);
-    }
-  }
-  auto stage = [&](int t, int buf) {
-    const Tile T = tile_of(t, g);
-    const uint32_t sa = sh + buf * buf_bytes, sg = sa + W::ABYTES;
-    for (int idx = tid; idx < HROWS * CG; idx += CTHREADS) {
-      const int cg = idx % CG, h = idx / CG, dy = h / HPL, rem = h - dy * HPL, xx = rem / HZ, zz = rem - xx * HZ;
-      const int yy = T.y + dy - 1, xg = T.x0 + xx - 1, zg = T.z0 + zz - 1;
-      const bool ok = (unsigned)yy < (unsigned)g.ny && (unsigned)xg < (unsigned)g.nx && (unsigned)zg < (unsigned)g.nz;
-      const __nv_bfloat16* src = ok ? g.a + g.a_off + ((size_t)(yy * g.nx + xg) * g.nz + zg) * g.a_stride + cg * 8 : g.a;
-      umma::cp16(sa + (dy * CG + cg) * GP + rem * 16, src, ok ? 16u : 0u);
-    }
-    for (int idx = tid; idx < 128 * NG; idx += CTHREADS) {
-      const int ng = idx % NG, r = idx / NG, x = T.x0 + (r >> 3), z = T.z0 + (r & 7);
-      const bool ok = x < g.nx && z < g.nz;
-      const __nv_bfloat16* src = ok ? g.b + g.b_off + ((size_t)(T.y * g.nx + x) * g.nz + z) * g.b_stride + n_first + ng * 8 : g.b;
-      umma::cp16(sg + ng * 2048 + r * 16, src, ok ? 16u : 0u);
-    }
-  };
-  const int n = blockIdx.x < tiles ? (tiles - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
-  auto tile_at = [&](int it) { return blockIdx.x + it * gridDim.x; };
-  for (int k = 0; k < std::max(1, BUFS - 1); ++k) {
-    if (k < n) stage(tile_at(k), k);
-    umma::cp_commit();
-  }
-  umma::fence_before_sync();
-  __syncthreads();
-  umma::fence_after_sync();
-  const uint32_t tmem = tmem_slot;
-  const uint32_t idesc = umma::idesc_bf16(128, Nt, true, true);
-  bool failed = false;
-  for (int it = 0; it < n; ++it) {
-    umma::cp_wait<(BUFS > 2 ? BUFS - 2 : 0)>();
-    umma::fence_proxy_async_smem();
-    if (__syncthreads_or(failed)) break;
-    if (tid == 0) {
-      umma::fence_after_sync();
-      const uint32_t sa = sh + (it % BUFS) * buf_bytes, sg = sa + W::ABYTES;
-      for (int t9 = 0; t9 < 9; ++t9) {
-        const uint32_t a0 = sa + (uint32_t)((t9 / 3) * HZ + t9 % 3) * 16;
-#pragma unroll
-        for (int ch = 0; ch < W::CHUNKS; ++ch)
-#pragma unroll
-          for (int ks = 0; ks < 8; ++ks)  // 16 voxels: two z-runs
-            umma::mma_bf16(tmem + (t9 * W::CHUNKS + ch) * Nt, umma::smem_desc(a0 + ch * 16 * GP + ks * 2 * HZ * 16, HZ * 16, GP),
-                           umma::smem_desc(sg + ks * 256, 128, 2048), idesc, it + ks > 0 ? 1u : 0u);
-      }
-      umma::commit(&mbar[it % BUFS]);
-    }
-    const int nx = it + std::max(1, BUFS - 1);
-    if (nx < n) {
-      // the buffer of tile nx was last read by the MMAs of tile nx - BUFS
-      const int prev = nx - BUFS;
-      if (prev >= 0) failed = !umma::mbar_wait(&mbar[prev % BUFS], (prev / BUFS) & 1, CWAIT);
-      if (!failed) stage(tile_at(nx), nx % BUFS);
-    }
-    umma::cp_commit();
-  }
-  umma::cp_wait<0>();
-  if (n > 0 && !failed) failed = !umma::mbar_wait(&mbar[(n - 1) % BUFS], ((n - 1) / BUFS) & 1, CWAIT);
-  const bool any = __syncthreads_or(failed);
-  if (any) drain_failed(4);
-  umma::fence_after_sync();
-  // partial sums: row m of chunk ch is (dy, ci) = ((128 ch + m) / C, (128 ch + m) % C)
-  const uint32_t trow = tmem + ((uint32_t)(tid & 96) << 16);
-  for (int ch = 0; ch < W::CHUNKS; ++ch) {
-    const int m = ch * 128 + (tid & 127), dy = m / C, ci = m - dy * C;
-    for (int t9 = tid >> 7; t9 < 9; t9 += CPARTS)
-      for (int n0 = 0; n0 < Nt; n0 += 8) {
-        float v[8];
-        umma::tmem_ld8(trow + (t9 * W::CHUNKS + ch) * Nt + n0, v);
-        if (any) continue;
-        float* dst = nullptr;
-        if (m < 3 * C) dst = g.outf + ((size_t)blockIdx.x * 27 * C + (size_t)(dy * 9 + t9) * C + ci) * g.N + n_first + n0;
-        else if (W::ONES && m == 3 * C && t9 == 0) dst = bias_part + (size_t)blockIdx.x * g.N + n_first + n0;
-        if (!dst) continue;
-        *reinterpret_cast<float4*>(dst) = n > 0 ? make_float4(v[0], v[1], v[2], v[3]) : make_float4(0.f, 0.f, 0.f, 0.f);
-        *reinterpret_cast<float4*>(dst + 4) = n > 0 ? make_float4(v[4], v[5], v[6], v[7]) : make_float4(0.f, 0.f, 0.f, 0.f);
-      }
-  }
-  umma::fence_before_sync();
-  __syncthreads();
-  if (warp == 0) umma::tmem_dealloc(tmem, ncols);
-}
-
-static int wgrad_slice(int C, int N) { return C <= 32 ? std::min(32, N) : 16; }
-
-int wgrad3_blocks(const GemmArgs& g) {
-  const int tiles = ((g.nz + 7) / 8) * ((g.nx + 15) / 16) * g.ny, slices = g.N / wgrad_slice(g.a_c, g.N);
-  return std::min(tiles, std::max(1, 152 * (g.a_c <= 16 ? 2 : 1) / slices));
-}
-
-bool wgrad3_fits(const GemmArgs& g) {
-  const int C = g.a_c;
-  return (C == 8 || C == 16 || C == 32 || C == 64 || C == 128) && (g.N == 16 || g.N % 32 == 0);
-}
-
-bool wgrad3_sums_bias(int C) { return C < 128; }
-
-cudaError_t launch_wgrad3(const GemmArgs& g, float* bias_part, cudaStream_t s) {
-  if (!wgrad3_fits(g)) return cudaErrorNotSupported;
-  const int C = g.a_c, Nt = wgrad_slice(C, g.N);
-  const int tiles = ((g.nz + 7) / 8) * ((g.nx + 15) / 16) * g.ny;
-  const dim3 grid(wgrad3_blocks(g), g.N / Nt);
-  auto go = [&](auto kern, size_t abytes, int bufs, int chunks) -> cudaError_t {
-    // the last chunk's M blocks may run past the planes: their rows are not used, but must be readable
-    const size_t reach = (size_t)chunks * 16 * HPL * 16 + 2 * HZ * 16 + 1024;
-    const size_t smem = (size_t)(bufs - 1) * (abytes + (size_t)(Nt / 8) * 2048) + std::max(abytes + (size_t)(Nt / 8) * 2048, reach);
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    kern<<<grid, CTHREADS, smem, s>>>(g, tiles, Nt, bias_part);
-    return cudaGetLastError();
-  };
-  switch (C) {
-    case 8: return go(k_wgrad3<8>, Wg<8>::ABYTES, Wg<8>::BUFS, Wg<8>::CHUNKS);
-    case 16: return go(k_wgrad3<16>, Wg<16>::ABYTES, Wg<16>::BUFS, Wg<16>::CHUNKS);
-    case 32: return go(k_wgrad3<32>, Wg<32>::ABYTES, Wg<32>::BUFS, Wg<32>::CHUNKS);
-    case 64: return go(k_wgrad3<64>, Wg<64>::ABYTES, Wg<64>::BUFS, Wg<64>::CHUNKS);
-    default: return go(k_wgrad3<128>, Wg<128>::ABYTES, Wg<128>::BUFS, Wg<128>::CHUNKS);
-  }
 }
 
 }  // namespace ig

@@ -52,12 +52,6 @@ cudaError_t launch(int am, int bm, int em, const GemmArgs& g, dim3 grid, cudaStr
 // block before tap 26 for a_c = 8) from a staged input halo with the taps as shifted shared-memory descriptors, BF16 output;
 // cudaErrorNotSupported for 256 input channels, which launch() serves with weights [N][27 a_c]
 cudaError_t launch_conv3(const GemmArgs& g, cudaStream_t s);
-// 3x3x3 weight gradient (A_WG_CONV3, B_WG_ROWS operands): partial sums outf[block][27 a_c][N] of
-// wgrad3_blocks(g) blocks, and the column sums of b in bias_part[block][N] where wgrad3_sums_bias(a_c)
-bool wgrad3_fits(const GemmArgs& g);
-bool wgrad3_sums_bias(int a_c);
-int wgrad3_blocks(const GemmArgs& g);
-cudaError_t launch_wgrad3(const GemmArgs& g, float* bias_part, cudaStream_t s);
 // first failure code recorded by any launch (0: none); synchronises s
 int read_error(cudaStream_t s);
 
