@@ -413,10 +413,12 @@ static int build_bwd_table(spdhg_ctx* ctx, cudaStream_t s) {
   if (e == cudaSuccess) e = cudaMemcpyAsync(tot.data(), totals, V * sizeof(unsigned), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(&hbad, bad, sizeof(unsigned), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  if (e != cudaSuccess) {
+  auto failed = [&]() {
     release();
+    ctx->bwd_table = -1;  // the same call fails again
     return fail(ctx, SPDHG_ERR_CUDA, std::string("backprojector table: ") + cudaGetErrorString(e));
-  }
+  };
+  if (e != cudaSuccess) return failed();
   std::vector<unsigned> base(V);
   uint64_t total = 0;
   for (size_t v = 0; v < V; ++v) {
@@ -444,8 +446,14 @@ static int build_bwd_table(spdhg_ctx* ctx, cudaStream_t s) {
   e = cudaMemcpyAsync(totals, base.data(), V * sizeof(unsigned), cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) e = backward_table_fill(g, starts, totals, ctx->bwd_items, ctx->bwd_hdr, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  if (e != cudaSuccess) {
+    ctx_free(ctx, ctx->bwd_items);
+    ctx_free(ctx, ctx->bwd_hdr);
+    ctx->bwd_items = nullptr;
+    ctx->bwd_hdr = nullptr;
+    return failed();
+  }
   release();
-  if (e != cudaSuccess) return fail(ctx, SPDHG_ERR_CUDA, std::string("backprojector table: ") + cudaGetErrorString(e));
   ctx->bwd_table = 1;
   ++ctx->graph_gen;
   return status;
@@ -1332,9 +1340,9 @@ int spdhg_osem(spdhg_ctx* ctx, const spdhg_params* params, int mlem, float* x_in
       a.out = ctx->em_sens + (size_t)i * N;
       CK(launch_backward(ctx->dg, sub, BWD_OUT, a, s));
     }
-    ctx->em_sens_kind = kind;
     if (!mlem)
       if (int st = build_bwd_table(ctx, s)) return st;
+    ctx->em_sens_kind = kind;
   }
   // the iterate: u0 from the caller, or ones (Eq. EQU:MLEM needs a positive start)
   float* u = ctx->x[0];

@@ -96,11 +96,13 @@ void backward_layout(DevGeom& g, const SegDev* seg, CompDev* comp, std::vector<i
     g.bw_buf = std::max(g.bw_buf, (g.bw_rows * b.slots + 3) & ~3);
   }
   g.bw_nb = (int)batches.size();
-  // several views per stage where their rows are short: fewer barriers, fuller records
+  // several views per stage where their rows are short (fewer barriers, fuller records) and their pair
+  // lists fit: with many bins per pixel the lists, not the rows, take the room
   g.bw_views = 1;
   if (g.bw_nb == 1) {
     const int most = g.bins ? g.V : (g.V + g.m - 1) / g.m;
-    const int fit = std::max(1, std::min(16, room / batches[0].slots));
+    const int lists = (int)(kPairBytes / ((size_t)kBwdWarps * g.bw_cpw * g.bw_cand * sizeof(PixItem)));
+    const int fit = std::max(1, std::min(std::min(16, lists), room / batches[0].slots));
     const int stages = (most + fit - 1) / fit;
     g.bw_views = (most + stages - 1) / stages;
     g.bw_buf = (g.bw_views * g.bw_rows * batches[0].slots + 3) & ~3;

@@ -10,6 +10,8 @@ namespace spdhg {
 
 constexpr int kBwdWarps = 8;      // warps per block: 2 in x, 4 in y, CPW columns in x each
 constexpr int kBwdFill = 32;      // item records a warp holds at a time (one per lane)
+constexpr size_t kPairBytes = 48 * 1024;   // most of the warps' pair lists: what a kernel has without opting in
+constexpr size_t kBwdMaxSmem = 220 * 1024;
 constexpr float kBinMargin = 0.01f;   // radial bins: covers the FP32 rounding of the footprint ends
 
 // A (bin, pixel interval) pair: the LOR lines of radial bin r of one view of the stage that cross
@@ -512,6 +514,21 @@ __global__ void __launch_bounds__(kBwdWarps * 32) k_bwd_items(const __grid_const
 // launches
 // ---------------------------------------------------------------------------------------
 
+// Bytes of the warps' pair lists.  backward_layout chooses the views per stage so that they stay within
+// kPairBytes, with any geometry: neither kernel then needs more shared memory than it may ask for.
+inline size_t bwd_pair_bytes(const DevGeom& g) {
+  return ((size_t)kBwdWarps * g.bw_cpw * g.bw_views * g.bw_cand * sizeof(PixItem) + 15) & ~(size_t)15;
+}
+
+// Dynamic shared memory of k_backward (its carve-up in order): records, wide offsets, pairs, sums, staging.
+inline size_t bwd_smem(const DevGeom& g, int nt, int zk, bool single, bool tab, bool mashed) {
+  size_t smem = (size_t)kBwdWarps * kBwdFill * 16 * (1 + (zk + 3) / 4 * (mashed && nt > 2 ? 2 : 1));
+  if (nt > 3) smem += (size_t)kBwdWarps * kBwdFill * 4;
+  if (!tab) smem += bwd_pair_bytes(g);
+  if (!single) smem += (size_t)kBwdWarps * g.bw_cpw * zk * 128;
+  return smem + (size_t)g.bw_buf * sizeof(float);
+}
+
 inline dim3 bwd_tiles(const DevGeom& g) { return dim3((g.nx + 2 * g.bw_cpw - 1) / (2 * g.bw_cpw), (g.ny + 3) / 4); }
 
 // view groups of a subset (the same for all subsets, whose view counts differ by at most one)
@@ -523,12 +540,8 @@ inline int bwd_groups(const DevGeom& g, int subset) {
 template <int NT, int ZK, int CPW, bool SINGLE, bool TAB, bool MASHED>
 cudaError_t bwd_run(const DevGeom& g, int subset, int mode, const BwdArgs& a, cudaStream_t s) {
   const int groups = bwd_groups(g, subset);
-  size_t smem = (size_t)kBwdWarps * kBwdFill * 16 * (1 + (ZK + 3) / 4 * mask_sets<NT, MASHED>());
-  if (NT > 3) smem += (size_t)kBwdWarps * kBwdFill * 4;
-  if (!TAB) smem += ((size_t)kBwdWarps * CPW * g.bw_views * g.bw_cand * sizeof(PixItem) + 15) & ~(size_t)15;
-  if (!SINGLE) smem += (size_t)kBwdWarps * CPW * ZK * 128;
-  smem += (size_t)g.bw_buf * sizeof(float);
-  if (smem > 220 * 1024) return cudaErrorInvalidValue;
+  const size_t smem = bwd_smem(g, NT, ZK, SINGLE, TAB, MASHED);
+  if (smem > kBwdMaxSmem) return cudaErrorInvalidValue;
   auto kern = k_backward<NT, ZK, CPW, SINGLE, TAB, MASHED>;
   cudaError_t e = allow_dynamic_smem(kern, smem);
   if (e != cudaSuccess) return e;
@@ -571,7 +584,7 @@ cudaError_t backward_items_nt(const DevGeom& g, int pass, unsigned short* cnt, u
                               const unsigned* stage_base, float4* items, int2* hdr, cudaStream_t s) {
   const int groups = bwd_groups(g, 0);
   const dim3 t = bwd_tiles(g), grid(t.x, t.y, g.m * groups);
-  const size_t smem = (size_t)kBwdWarps * g.bw_cpw * g.bw_views * g.bw_cand * sizeof(PixItem);
+  const size_t smem = bwd_pair_bytes(g);
   auto go = [&](auto kern) {
     kern<<<grid, kBwdWarps * 32, smem, s>>>(g, groups, cnt, bad, starts, stage_base, items, hdr);
     return cudaGetLastError();
