@@ -84,10 +84,27 @@ __device__ __forceinline__ unsigned lane_range(int off, int len) {
   return m;
 }
 
-// Item record word: 4 x (staged offset + kOffBias) | (taps - 1); the bias keeps it non-negative.
-// The words of step-2 components are marked kStep2; their low bits are a parity and kMoreTaps.
+// Item record word: 4 x (staged offset + kOffBias) | (taps - 1).  The words of step-2 components are marked
+// kStep2; their low bits are a parity and kMoreTaps.
 constexpr int kOffBias = 256;
 constexpr unsigned kStep2 = 1u << 31, kMoreTaps = 2u;
+
+// Word of an item whose tap 0 meets, in lane b, slot b + jp of a run of len lanes from row_slot on; `lanes`
+// lanes (at most kOffBias) look at it, `taps` of its taps have a weight.  A component's planes may lie
+// wholly above or below the image's slices: then no lane is in the run, the offset does not matter and may be
+// too low for the bias, so that the word would carry the mark of a step-2 component.  Such an item becomes
+// one without lanes at offset 0.  jp and len are what the masks are made of: lanes b with 0 <= b + jp < len,
+// and with 0 <= b + jp + 2 < len for the taps above the second of a step-2 component.
+__host__ __device__ inline unsigned item_word(int row_slot, int& jp, int& len, int taps, int lanes, int pad, bool step2) {
+  if (step2) jp -= pad - 1;  // tap 1 of lane b meets plane b + jp of the component, if that is even
+  const bool more = step2 && taps > 2;
+  if (jp >= len || jp + (more ? 2 : 0) <= -lanes) {
+    jp = len = 0;
+    taps = 1;
+  }
+  if (!step2) return (unsigned)(4 * (row_slot + jp + kOffBias) | (taps - 1));
+  return (unsigned)(4 * (row_slot + (jp >> 1) + kOffBias) | (jp & 1)) | (taps > 2 ? kMoreTaps : 0u) | kStep2;
+}
 
 // lane masks per record: one set, and one for the taps above the second of a step-2 component
 template <int NT, bool MASHED>
@@ -360,12 +377,9 @@ __global__ void __launch_bounds__(kBwdWarps * 32, ZK <= 4 ? 4 : 3)
 #pragma unroll
         for (int k = 1; k < NT; ++k)
           if (L[k] != 0.f) nt = k + 1;
-        int word = 4 * (row_slot + jp + kOffBias) | (nt - 1);
         const bool step2 = MASHED && smask;
-        if (step2) {
-          jp -= PAD - 1;  // tap 1 of lane b meets plane b + jp of the component, if that is even
-          word = (4 * (row_slot + (jp >> 1) + kOffBias) | (jp & 1)) | (nt > 2 ? (int)kMoreTaps : 0) | (int)kStep2;
-        }
+        // (without marks in the words an item of empty masks is harmless at any offset)
+        const int word = MASHED ? (int)item_word(row_slot, jp, len, nt, 32 * ZK, PAD, step2) : 4 * (row_slot + jp + kOffBias) | (nt - 1);
         recA[lane] = make_float4(L[0], L[1], L[2], NT > 3 ? L[3] : __int_as_float(word));
         if (NT > 3) recO[lane] = word;
         auto masks = [&](uint4* to, int off) {
@@ -381,7 +395,7 @@ __global__ void __launch_bounds__(kBwdWarps * 32, ZK <= 4 ? 4 : 3)
         };
         masks(recM + lane * MR, jp);
         if constexpr (mask_sets<NT, MASHED>() > 1) {
-          if (step2 && nt > 2) masks(recM + lane * MR + MQ, jp + 2);
+          if (word & (int)kStep2) masks(recM + lane * MR + MQ, jp + 2);
         }
       }
       base = it;

@@ -5,6 +5,8 @@
   opting in and the whole launch within the limit of k_backward.
 * Its staged rows and candidate bins cover every bin whose lines cross a pixel of the tile, by
   brute force over the kernel's FP32 formulas and the exact footprints.
+* An item's record word names its kind and the staged slots of its lanes for components whose planes lie
+  inside, across and wholly outside the image's slices.
 """
 import ctypes
 import math
@@ -39,11 +41,14 @@ extern "C" void layout(const int* in, float inv, int n_seg, const int* seg_n, in
   out[6] = (long long)bwd_smem(g, g.taps, zk, false, false, g.bw_step2);
   out[7] = kBwdMaxSmem;
 }
+extern "C" unsigned word(int row_slot, int* jp, int* len, int taps, int lanes, int pad, int step2) {
+  return item_word(row_slot, *jp, *len, taps, lanes, pad, step2 != 0);
+}
 """
 
 
 @pytest.fixture(scope="module")
-def layout(tmp_path_factory):
+def helper(tmp_path_factory):
     lib = _build_ext.build()
     d = tmp_path_factory.mktemp("layout")
     src, so = str(d / "layout.cu"), str(d / "layout.so")
@@ -52,7 +57,12 @@ def layout(tmp_path_factory):
     subprocess.run([_build_ext._nvcc(), *_build_ext.ARCH, "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr",
                     "-shared", "-I", _build_ext.CSRC, src, lib, "-o", so,
                     "-Xlinker", f"-rpath={os.path.dirname(lib)}"], check=True, capture_output=True)
-    fn = ctypes.CDLL(so).layout
+    return ctypes.CDLL(so)
+
+
+@pytest.fixture(scope="module")
+def layout(helper):
+    fn = helper.layout
 
     def run(nx, ny, nz, inv, views, subsets, taps, seg_n, comps, bins=0):
         a = lambda v: np.ascontiguousarray(v, np.int32).ctypes.data_as(ctypes.POINTER(ctypes.c_int))
@@ -117,3 +127,32 @@ def test_staged_rows_and_candidates_cover_every_footprint(layout, n, inv):
         some = e_lo <= e_hi
         assert (np.maximum(lo, r_min)[some] <= e_lo[some]).all()
         assert (np.minimum(hi, r_max)[some] >= e_hi[some]).all()
+
+
+@pytest.mark.parametrize("step2", [0, 1])
+@pytest.mark.parametrize("lanes", [32, 96, 256])
+def test_record_words_name_their_kind_and_slots(helper, lanes, step2):
+    helper.word.restype = ctypes.c_uint
+    b = np.arange(lanes)
+    for pad in range(4):
+        for taps in range(1, pad + 2):
+            for row_slot in (0, 1, 5000):
+                for n in (1, 2, 31, 300):
+                    for jp0 in [*range(-lanes - 6, 8), *range(n - 4, n + 4), -9000, -1000, -300, 300, 9000]:
+                        jp, ln = ctypes.c_int(jp0), ctypes.c_int(n)
+                        w = helper.word(row_slot, ctypes.byref(jp), ctypes.byref(ln), taps, lanes, pad, step2)
+                        assert (w >> 31) == step2
+                        off = ((w & 0x7FFFFFFF) >> 2) - 256
+                        at = b + jp0 - (pad - 1 if step2 else 0)  # the run's lane of tap 0 (step 2: of taps 0 and 1)
+                        sets = (0, 2) if step2 and taps > 2 else (0,)
+                        seen = False
+                        for add in sets:
+                            want, got = (at + add >= 0) & (at + add < n), (b + jp.value + add >= 0) & (b + jp.value + add < ln.value)
+                            assert (want == got).all()
+                            if not want.any():
+                                continue
+                            seen = True
+                            slot = off + (((b + (w & 1)) >> 1) + add // 2 if step2 else b)
+                            assert (slot == row_slot + ((at + add) // 2 if step2 else at))[want].all()
+                        more = (w & 3) if not step2 else (w >> 1) & 1
+                        assert more == ((taps - 1 if not step2 else taps > 2) if seen else 0)
