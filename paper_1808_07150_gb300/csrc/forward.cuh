@@ -168,7 +168,9 @@ __device__ __forceinline__ void forward_epilogue(const DevGeom& g, const FwdArgs
 // enough for every tap of every plane of the segments (the axial bound of the geometry, so no plane
 // needs a range test), and its axial taps computed while chunk c is accumulated.  One tap record
 // serves all words of a task, packed FP32 FMAs accumulate two words.  Mashed geometries sum the
-// components of the segment one after the other, each kept by the planes that include it.  When a
+// components of the segment one after the other, each kept by the planes that include it, and a chunk's
+// component sums before they join the bin's (each joining by itself, a bin of nine components came to 2.7
+// units (2^-24) from its FP64 value instead of 1.3, relative L2; 38.7 -> 39.1 us).  When a
 // line has few tasks, egroups warps share each, warp group k taking the entries k, k + egroups, ...
 // of every chunk; group 0 adds the other groups' sums in group order.  When several row parts share
 // a line, each writes partial plane sums and the last one to finish reduces them in a fixed order.
@@ -179,7 +181,7 @@ __device__ __forceinline__ void forward_epilogue(const DevGeom& g, const FwdArgs
 // GB300, per launch: 344 x 344 x 127 voxels, one view of 344 x 837 bins, 92 -> 63 us; 171 x 171 x 92,
 // 12-13 views x 250 planes, 128 -> 77 us (115 with a warp per column of 4-byte copies); 128 x 128 x 64,
 // 8-9 views, three mashed components, 58 -> 39 us.  Blocks with entry groups are bounded to 56
-// registers (three blocks of 12 warps per SM; 39 against 43 us at 64), the others to 85 (63 against
+// registers (three blocks of 12 warps per SM; 39 against 43 us at 64), the others to 80 (63 against
 // 65 us at the mMR scale).
 template <int NT, int MODE, bool GROUPS, bool MASHED>
 __global__ void __launch_bounds__(kFwdMaxWarps * 32, GROUPS ? 3 : 2)
@@ -331,15 +333,26 @@ __global__ void __launch_bounds__(kFwdMaxWarps * 32, GROUPS ? 3 : 2)
     const int ne = min(chunk, n_ent - (c << csh));
     const float* xl = xs + (buf << csh) * xs_stride + q;
     const int rb = (buf * ncomp_tab + sd.c0 - c_lo) << csh;
-    const int nc = MASHED ? sd.nc : 1;
-    for (int ci = 0; ci < nc; ++ci) {
+    if (!MASHED) {
       float2 s[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-      gather_words<NT>(words, xl, recA + rb + (ci << csh), recB + rb + (ci << csh), eg, ne, egroups, s);
-      const bool all = !MASHED;
-      acc[0] += all || (incl[0] >> ci) & 1u ? s[0].x : 0.f;
-      acc[1] += all || (incl[1] >> ci) & 1u ? s[0].y : 0.f;
-      acc[2] += all || (incl[2] >> ci) & 1u ? s[1].x : 0.f;
-      acc[3] += all || (incl[3] >> ci) & 1u ? s[1].y : 0.f;
+      gather_words<NT>(words, xl, recA + rb, recB + rb, eg, ne, egroups, s);
+      acc[0] += s[0].x;
+      acc[1] += s[0].y;
+      acc[2] += s[1].x;
+      acc[3] += s[1].y;
+    } else {
+      // the components' sums of the chunk are added first
+      float sum[4] = {0.f, 0.f, 0.f, 0.f};
+      for (int ci = 0; ci < sd.nc; ++ci) {
+        float2 s[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+        gather_words<NT>(words, xl, recA + rb + (ci << csh), recB + rb + (ci << csh), eg, ne, egroups, s);
+        sum[0] += (incl[0] >> ci) & 1u ? s[0].x : 0.f;
+        sum[1] += (incl[1] >> ci) & 1u ? s[0].y : 0.f;
+        sum[2] += (incl[2] >> ci) & 1u ? s[1].x : 0.f;
+        sum[3] += (incl[3] >> ci) & 1u ? s[1].y : 0.f;
+      }
+#pragma unroll
+      for (int w = 0; w < 4; ++w) acc[w] += sum[w];
     }
     __syncthreads();
   }
