@@ -22,7 +22,11 @@ struct Comp {
     two_prod(a, b, p, e);
     add(p, e);
   }
-  __device__ __forceinline__ float value() const { return s + c; }
+  // s is the plain sum; where it has left the finite numbers the errors are NaN and s stands alone
+  __device__ __forceinline__ float value() const {
+    const float v = s + c;
+    return v == v ? v : s;
+  }
 };
 
 bool flat_geometry(const DevGeom& g) { return g.nz == 1 && g.P == 1 && g.n_comp == 1 && g.taps == 1; }
