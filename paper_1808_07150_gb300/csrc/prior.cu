@@ -114,7 +114,7 @@ __global__ void __launch_bounds__(kPriorWarps * 32, 1) k_prior(March m, PriorArg
   float *ox = a.q_out + (size_t)m.kx * N, *oy = a.q_out + (size_t)m.ky * N, *oz = a.q_out + (size_t)m.kz * N;
   const float *X = a.x_in, *V = a.side;
   // Dead lanes read a live voxel (their duals are never used), and a neighbour past the end is the
-  // voxel itself (a zero difference), so the loads need no tests.
+  // voxel itself, so the loads need no tests.  The difference there is 0 also where the voxel is not finite.
   const int dx = hx ? sx : 0, dz1 = hz ? 1 : 0;
   int i = ys * sy + (live ? ix * sx + iz : 0);
   // this row: x and v of the voxel and of its neighbours in y, x, z; q, z, T
@@ -143,7 +143,7 @@ __global__ void __launch_bounds__(kPriorWarps * 32, 1) k_prior(March m, PriorArg
     }
     const float n0 = qx[j], n1 = qy[j], n2 = qz[j], nzo = a.z[j], nTo = a.T[j];
     float b[3], qn[3];
-    const float gr[3] = {xr - xc, xd - xc, xu - xc}, gv[3] = {vr - vc, vd - vc, vu - vc}, qo[3] = {q0, q1, q2};
+    const float gr[3] = {hx ? xr - xc : 0.f, iy < ny - 1 ? xd - xc : 0.f, hz ? xu - xc : 0.f}, gv[3] = {vr - vc, vd - vc, vu - vc}, qo[3] = {q0, q1, q2};
     dual_update<KIND>(a, gr, gv, qo, b, qn);
     *bx = b[0];
     if (lane == 31) *bz = b[2];
@@ -248,7 +248,7 @@ __global__ void __launch_bounds__(kTgvWarps * 32, 1) k_tgv0(March m, TgvArgs a, 
       nzw[k] = a.zw[off[k] + j];
     }
     float b[3], qn[3], qa[3];
-    const float gr[3] = {ur - uc, ud - uc, uu - uc};
+    const float gr[3] = {hx ? ur - uc : 0.f, iy < ny - 1 ? ud - uc : 0.f, hz ? uu - uc : 0.f};
 #pragma unroll
     for (int k = 0; k < 3; ++k) qa[k] = fmaf(a.sigma, gr[k] - wv[k], qo[k]);
     const float nrm = sqrtf(qa[0] * qa[0] + qa[1] * qa[1] + qa[2] * qa[2]);

@@ -32,3 +32,22 @@ def test_flat_projections_of_an_infinite_value():
             torch.cuda.synchronize()
             assert bool(meets.any()) and bool((got[meets] == float("inf")).all())
             assert torch.equal(got[~meets], rest[~meets])
+
+
+@pytest.mark.parametrize("sc", [_flat(), synth.tiny_3d(n_subsets=2)], ids=lambda s: s.name)
+@pytest.mark.parametrize("kind", ["tv", "dtv", "atv", "tgv"])
+def test_prior_duals_beyond_the_last_voxel(sc, kind):
+    """The last voxel has no neighbour in any direction: its gradient is 0 whatever it holds."""
+    import paper_1808_07150_gb300 as pkg
+    import torch
+    d, _ = problem(sc, side=kind == "dtv")
+    x0 = np.ones(sc.image_shape, np.float32)
+    x0[-1, -1, -1] = np.inf
+    q = torch.full((3 * sc.n_voxels,), 7.0, device="cuda")
+    with pkg.Context(sc) as ctx:
+        upload(ctx, d)
+        ctx.spdhg_setup(pkg.make_params(kind, alpha=0.08, alpha0=0.2, alpha1=0.1), dev(x0))
+        ctx.spdhg_iterate(np.array([sc.n_subsets], np.int32))  # the (first) prior block
+        ctx.spdhg_get("q", q)
+        torch.cuda.synchronize()
+    assert (host(q).reshape(3, -1)[:, -1] == 0.0).all()
