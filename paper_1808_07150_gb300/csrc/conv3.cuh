@@ -95,13 +95,14 @@ __device__ __forceinline__ void load_bias(const GemmArgs& g, int n_first, int Nt
 // ------------------------------------------------------------------------------------------
 
 constexpr int kHaloBufs = 3;
+constexpr int kZeroBytes = (15 * HZ + 8) * 16;  // 16 core matrices at the halo's distance
 
 template <int C>
 __global__ void __launch_bounds__(CTHREADS) k_conv3_halo(const __grid_constant__ GemmArgs g, int tiles, int Nt) {
   constexpr int CG = C / 8;                            // channel groups
   constexpr uint32_t GP = HROWS * 16;                  // bytes of a group's halo
   constexpr int PIECES = (HROWS * CG + CTHREADS - 1) / CTHREADS;
-  constexpr int TAPS = C == 8 ? 28 : 27;               // weight blocks (8 channels: taps 0 .. 25, zeros, tap 26)
+  constexpr int TAPS = C == 8 ? 28 : 27;               // weight blocks (8 channels: a zero block at the end)
   extern __shared__ __align__(1024) unsigned char smem[];
   __shared__ uint64_t mbar[2];
   __shared__ uint32_t tmem_slot;
@@ -118,6 +119,9 @@ __global__ void __launch_bounds__(CTHREADS) k_conv3_halo(const __grid_constant__
     umma::fence_mbar_init();
   }
   load_bias(g, n_first, Nt, sbias);
+  if (C == 8)  // the zero operand after the weights
+    for (int i = tid; i < kZeroBytes / 16; i += CTHREADS)
+      *reinterpret_cast<uint4*>(smem + kHaloBufs * halo + TAPS * tapb + 16 * i) = make_uint4(0u, 0u, 0u, 0u);
   // weights: [tap][n / 8][c / 8] core matrices; the slice's rows of a tap are contiguous
   for (int i = tid; i < TAPS * (int)(tapb >> 4); i += CTHREADS) {
     const int tap = i / (int)(tapb >> 4), k = i - tap * (int)(tapb >> 4);
@@ -160,12 +164,12 @@ __global__ void __launch_bounds__(CTHREADS) k_conv3_halo(const __grid_constant__
       const uint32_t a0 = sh + (it % kHaloBufs) * halo, d = tmem + (it & 1) * Nt;
       if (C == 8) {
         // a K step holds two taps; the distance of their starts is the leading-dimension offset.  The
-        // last step pairs tap 26 with tap 25 under zero weights (no read leaves the halo)
+        // last step pairs tap 26 with zeros (a voxel under a zero weight would spread infinities as NaN)
 #pragma unroll
         for (int i = 0; i < 14; ++i) {
-          const int t0 = i < 13 ? 2 * i : 25, t1 = i < 13 ? 2 * i + 1 : 26;
-          umma::mma_bf16(d, umma::smem_desc(a0 + tap_off(t0), tap_off(t1) - tap_off(t0), HZ * 16),
-                         umma::smem_desc(sb + 2 * i * tapb, tapb, 128), idesc, i > 0 ? 1u : 0u);
+          const uint32_t t0 = a0 + tap_off(2 * i), t1 = i < 13 ? a0 + tap_off(2 * i + 1) : sb + TAPS * tapb;
+          umma::mma_bf16(d, umma::smem_desc(t0, t1 - t0, HZ * 16), umma::smem_desc(sb + 2 * i * tapb, tapb, 128), idesc,
+                         i > 0 ? 1u : 0u);
         }
       } else {
 #pragma unroll
@@ -295,7 +299,8 @@ cudaError_t launch_conv3(const GemmArgs& g, cudaStream_t s) {
     return cudaGetLastError();
   };
   if (C <= 32) {
-    const size_t smem = (size_t)kHaloBufs * (C / 8) * HROWS * 16 + (size_t)(C == 8 ? 28 : 27) * Nt * C * 2;
+    const size_t smem = (size_t)kHaloBufs * (C / 8) * HROWS * 16 +
+                        (C == 8 ? (size_t)28 * Nt * 16 + kZeroBytes : (size_t)27 * Nt * C * 2);
     const int per_sm = std::max(1, std::min(4, (int)(220 * 1024 / (smem + 1024)))), slices = g.N / Nt;
     const dim3 grid(std::min(tiles, std::max(1, 152 * per_sm / slices)), slices);
     if (C == 8) return go(k_conv3_halo<8>, grid, smem, tiles, Nt);

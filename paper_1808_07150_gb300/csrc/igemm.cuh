@@ -49,7 +49,7 @@ struct GemmArgs {
 
 cudaError_t launch(int am, int bm, int em, const GemmArgs& g, dim3 grid, cudaStream_t s);
 // 3x3x3 convolution (A_CONV3 operands; B = weights [tap][N / 8][a_c / 8][8][8], a zero
-// block before tap 26 for a_c = 8) from a staged input halo with the taps as shifted shared-memory descriptors, BF16 output;
+// block after them for a_c = 8) from a staged input halo with the taps as shifted shared-memory descriptors, BF16 output;
 // cudaErrorNotSupported for 256 input channels, which launch() serves with weights [N][27 a_c]
 cudaError_t launch_conv3(const GemmArgs& g, cudaStream_t s);
 // first failure code recorded by any launch (0: none); synchronises s

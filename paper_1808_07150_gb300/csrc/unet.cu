@@ -235,8 +235,7 @@ __global__ void k_bf16_conv3(const float* __restrict__ w, int cin, int cout, bf1
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     const int ci = i % cin, tap = (i / cin) % 27, co = i / (27 * cin);
     const bf16 h = __float2bfloat16_rn(w[i]);
-    const int pos = cin == 8 && tap == 26 ? 27 : tap;  // 8 channels: zeros at 26
-    wf[cin > 128 ? i : pos * per_tap + core_at(co, ci, cin)] = h;
+    wf[cin > 128 ? i : tap * per_tap + core_at(co, ci, cin)] = h;
     wb[(26 - tap) * per_tap + core_at(ci, co, cout)] = h;
   }
 }
@@ -632,7 +631,7 @@ int unet_create(int levels, const int* channels, int ny, int nx, int nz, unet_ne
   A(zalloc(&net->v, off));
   for (Param& p : net->P)
     if (p.kind != 2) {
-      A(zalloc(&p.wf, p.n + (p.kind == 0 ? (size_t)p.cout * p.cin : 0)));  // conv3 of 8 channels: a zero tap
+      A(zalloc(&p.wf, p.n + (p.kind == 0 ? (size_t)p.cout * p.cin : 0)));  // conv3 of 8 channels: a zero block after the taps
       A(zalloc(&p.wb, p.n));
     }
   const int64_t V0 = net->V[0];

@@ -51,3 +51,27 @@ def test_prior_duals_beyond_the_last_voxel(sc, kind):
         ctx.spdhg_get("q", q)
         torch.cuda.synchronize()
     assert (host(q).reshape(3, -1)[:, -1] == 0.0).all()
+
+
+def test_first_convolution_of_an_infinite_voxel():
+    """Through one weight of 1 at tap (dy, dx, dz) the voxel at that distance becomes infinite, and the identity
+    layers behind it carry it to the prediction; every other tap's weight of 0 turns it into NaN, which ReLU clears."""
+    import torch
+    from oracle import unet as U
+    from paper_1808_07150_gb300 import learned
+    spec, shape, at = U.UNetSpec((16, 16)), (6, 20, 12), (3, 9, 6)
+    for tap in [(0, 0, 0), (1, 1, 1), (2, 2, 0), (2, 2, 1), (2, 2, 2)]:
+        p = {k: np.zeros(s, np.float32) for k, s in U.layer_shapes(spec)}
+        p["enc0a.W"][(0, 0) + tap] = 1.0
+        p["enc0b.W"][0, 0, 1, 1, 1] = 1.0
+        p["dec0a.W"][0, 16, 1, 1, 1] = 1.0
+        p["dec0b.W"][0, 0, 1, 1, 1] = 1.0
+        p["head.W"].flat[0] = 1.0
+        x = np.full(shape, 0.5, np.float32)
+        x[at] = np.inf
+        pred = torch.zeros(x.size, device="cuda")
+        with learned.UNet(shape, spec.channels) as net:
+            net.set_params(np.concatenate([p[k].ravel() for k, _ in U.layer_shapes(spec)]))
+            net.forward(dev(x), 1.0, pred)
+            out = host(pred).reshape(shape)
+        assert out[tuple(a - (t - 1) for a, t in zip(at, tap))] == np.inf, tap
