@@ -293,7 +293,7 @@ cudaError_t launch_conv3(const GemmArgs& g, cudaStream_t s) {
   if ((C != 8 && C != 16 && C != 32 && C != 64 && C != 128) || (g.N != 16 && g.N % 32)) return cudaErrorNotSupported;
   const int tiles = ((g.nz + 7) / 8) * ((g.nx + 15) / 16) * g.ny;
   auto go = [&](auto kern, dim3 grid, size_t smem, auto... args) -> cudaError_t {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_dynamic_smem(kern, smem);
     if (e != cudaSuccess) return e;
     kern<<<grid, CTHREADS, smem, s>>>(g, args...);
     return cudaGetLastError();

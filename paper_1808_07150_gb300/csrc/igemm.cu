@@ -24,6 +24,7 @@
 #include <algorithm>
 
 #include "igemm.cuh"
+#include "internal.cuh"
 #include "umma.cuh"
 
 namespace spdhg {
@@ -309,7 +310,7 @@ static cudaError_t launch_t(const GemmArgs& g, dim3 grid, cudaStream_t s) {
   const int NP = (g.N + 15) & ~15;
   const size_t smem = (size_t)STAGES * (BM * BK * 2 + (size_t)NP * BK * 2) + 1024;
   auto kern = k_igemm<AM, BMODE, EM>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_dynamic_smem(kern, smem);
   if (e != cudaSuccess) return e;
   kern<<<grid, THREADS, smem, s>>>(g);
   return cudaGetLastError();
