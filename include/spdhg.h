@@ -236,7 +236,8 @@ int spdhg_objective(spdhg_ctx* ctx, const float* x, int where, double out[3], vo
  * (host or device per `where`; NULL: ones) and the result is written back to it.  From `params`
  * only epochs, objective_every, target_gap / psi_star and x_star are used (as in spdhg_run; the
  * objective is the data term, no prior).  The sensitivity images P_i^T 1 are computed on the first
- * call after spdhg_set_data and kept (m x N floats for OSEM, N for MLEM).  The call replaces the
+ * call after spdhg_set_data and kept (m x N floats for OSEM, N for MLEM); OSEM then also builds the
+ * backprojector's item table (SPDHG_TUNE_BWD_TABLE) if the context has none.  The call replaces the
  * context's iterate: run spdhg_setup before further SPDHG iterations. */
 int spdhg_osem(spdhg_ctx* ctx, const spdhg_params* params, int mlem, float* x_inout, int where,
                spdhg_report* report, void* stream);
@@ -292,11 +293,12 @@ enum { SPDHG_TUNE_PRIOR_COLS = 0,   /* prior kernel: voxel columns per block, in
                                        over ceil(tasks / value) blocks */
        SPDHG_TUNE_PRIOR_STAGES = 4, /* accepted (3 or 4) without effect: the prior kernel has no
                                        shared-memory pipeline any more */
-       SPDHG_TUNE_BWD_TABLE = 5,    /* backprojector of the iterations: 0 reads its (pixel, bin,
-                                       segment) tap items from a table built by spdhg_setup when
-                                       it fits in 40 % of the free device memory (about 7 GB at
-                                       the mMR scale; same results bit for bit); 1 computes them in
-                                       the kernel */
+       SPDHG_TUNE_BWD_TABLE = 5,    /* backprojector of one subset (iterations, OSEM, spdhg_backproject):
+                                       0 reads its (pixel, bin, segment) tap items from a table built
+                                       by spdhg_setup or spdhg_osem when it fits in 40 % of the free
+                                       device memory (about 7 GB at the mMR scale; same results bit
+                                       for bit) and given back when a later allocation of the context
+                                       needs the memory; 1 computes them in the kernel */
        SPDHG_TUNE_FWD_GROUPS = 6,   /* forward projector: warps that share each plane task, each
                                        taking every k-th pixel entry of the line (1 .. 8; their
                                        partial sums are added in a fixed order); 0 = enough for

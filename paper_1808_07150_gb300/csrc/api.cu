@@ -15,17 +15,34 @@
 
 using namespace spdhg;
 
+// Frees the backprojector's table; the next spdhg_setup decides about it again.
+static void drop_bwd_table(spdhg_ctx* ctx) {
+  ctx_free(ctx, ctx->bwd_items);
+  ctx_free(ctx, ctx->bwd_hdr);
+  ctx->bwd_items = nullptr;
+  ctx->bwd_hdr = nullptr;
+  ctx->bwd_table = -1;
+  ++ctx->graph_gen;
+}
+
 // Device allocations of a context are charged to its memory limit (spdhg_set_memory_limit): one
 // that would take the context past the limit fails as an out-of-memory error, as the driver's
-// own would, and leaves the context usable.
+// own would, and leaves the context usable.  The backprojector's table only saves time, so it is given
+// back before an allocation fails.
 cudaError_t spdhg::ctx_malloc(spdhg_ctx* ctx, void** p, size_t bytes) {
-  if (ctx->mem_limit && ctx->mem_used + bytes > ctx->mem_limit) return cudaErrorMemoryAllocation;
-  const cudaError_t e = cudaMalloc(p, bytes);
-  if (e == cudaSuccess) {
-    ctx->mem_used += bytes;
-    ctx->mem_size[*p] = bytes;
+  for (;;) {
+    const bool over = ctx->mem_limit && ctx->mem_used + bytes > ctx->mem_limit;
+    const cudaError_t e = over ? cudaErrorMemoryAllocation : cudaMalloc(p, bytes);
+    if (e == cudaSuccess) {
+      ctx->mem_used += bytes;
+      ctx->mem_size[*p] = bytes;
+    }
+    if (e != cudaErrorMemoryAllocation || ctx->bwd_table != 1) return e;
+    cudaGetLastError();
+    const cudaError_t es = cudaDeviceSynchronize();  // kernels in flight may read the table
+    if (es != cudaSuccess) return es;
+    drop_bwd_table(ctx);
   }
-  return e;
 }
 
 void spdhg::ctx_free(spdhg_ctx* ctx, void* p) {
@@ -457,16 +474,6 @@ static int build_bwd_table(spdhg_ctx* ctx, cudaStream_t s) {
   ctx->bwd_table = 1;
   ++ctx->graph_gen;
   return status;
-}
-
-// Drops the table (a knob changed); the next spdhg_setup decides again.
-static void drop_bwd_table(spdhg_ctx* ctx) {
-  ctx_free(ctx, ctx->bwd_items);
-  ctx_free(ctx, ctx->bwd_hdr);
-  ctx->bwd_items = nullptr;
-  ctx->bwd_hdr = nullptr;
-  ctx->bwd_table = -1;
-  ++ctx->graph_gen;
 }
 
 int spdhg::forward_scratch(spdhg_ctx* ctx, int subset, FwdArgs& a, cudaStream_t s) {
