@@ -12,7 +12,7 @@ constexpr int kBwdWarps = 8;      // warps per block: 2 in x, 4 in y, CPW column
 constexpr int kBwdFill = 32;      // item records a warp holds at a time (one per lane)
 constexpr size_t kPairBytes = 48 * 1024;   // most of the warps' pair lists: what a kernel has without opting in
 constexpr size_t kBwdMaxSmem = 220 * 1024;
-constexpr int kSumItems = 12;     // records a column sums before the sum joins the others
+constexpr int kSumItems = 12;     // records of several taps a column sums before the sum joins the others
 constexpr float kBinMargin = 0.01f;   // radial bins: covers the FP32 rounding of the footprint ends
 
 // A (bin, pixel interval) pair: the LOR lines of radial bin r of one view of the stage that cross
@@ -208,7 +208,8 @@ __device__ __forceinline__ float ld_now(const float* p) {
 // (cp.async) as runs of planes (backward_layout), those of plain segments framed by NT - 1 zeros.  The
 // (bin, interval, component) items of a warp's columns are read from the table spdhg_setup builds
 // (TAB) or computed, one item per lane, and expanded to records in shared memory; a column's records are
-// then accumulated, kSumItems at a time, with lanes along z, 32 slices per register.  A record carries, per 32 slices, the mask of the lanes whose planes lie in the run: one AND decides a lane,
+// then accumulated with lanes along z, 32 slices per register; records of several taps kSumItems at a time.  A
+// record carries, per 32 slices, the mask of the lanes whose planes lie in the run: one AND decides a lane,
 // and words outside the run cost no shared-memory read.  In the last stage each column's x, z, T are
 // requested before its gather and its epilogue follows at once, so the epilogue traffic of some
 // warps overlaps the gathers of the others.  Between stages the sums rest in shared memory; with one
@@ -226,7 +227,8 @@ __device__ __forceinline__ float ld_now(const float* p) {
 // records, no masks) took the same time and room for fewer views.  Five blocks per SM spill.
 // Error of the mMR backprojection against FP64, and its time with computed items: one running sum per
 // column 9.10e-8, 96.5 us; sums of 8, 12, 16, 32 records 8.67, 8.83, 8.90, 8.99e-8 and 101.9, 99.6, 99.4, 98.3 us;
-// each item's taps summed first 8.92e-8, 110 us.  Columns of more records gain more (171 x 171 x 92: -9 %).
+// each item's taps summed first 8.92e-8, 110 us.  Columns of more records gain more.  With one tap a record rounds
+// once, so that one running sum is the closer one already (128 x 128 x 64, OSEM: 855 us, 875 in sums of twelve).
 template <int NT, int ZK, int CPW, bool SINGLE, bool TAB, bool MASHED>
 __global__ void __launch_bounds__(kBwdWarps * 32, ZK <= 4 ? 4 : 3)
     k_backward(const __grid_constant__ DevGeom g, int subset, int groups, int mode, const __grid_constant__ BwdArgs a) {
@@ -436,16 +438,23 @@ __global__ void __launch_bounds__(kBwdWarps * 32, ZK <= 4 ? 4 : 3)
       const int end = it + n;
       while (it < end) {
         if (it == filled) fill();
-        // Sums of few records at a time: added tap by tap to one running sum, the roundings of a column of
-        // many records grew with it (see above the kernel).
-        const int e = min(min(end, filled), it + kSumItems);
-        float part[ZK];
+        if constexpr (NT == 1) {
+          // one rounding per record, where a product added to a sum has two
+          const int e = min(end, filled);
+          gather_items<NT, ZK, MASHED>(buf, recA, recM, recO, it - base, e - base, bit, ac);
+          it = e;
+        } else {
+          // Sums of few records at a time: added tap by tap to one running sum, the roundings of a column
+          // of many records grew with it (see above the kernel).
+          const int e = min(min(end, filled), it + kSumItems);
+          float part[ZK];
 #pragma unroll
-        for (int k = 0; k < ZK; ++k) part[k] = 0.f;
-        gather_items<NT, ZK, MASHED>(buf, recA, recM, recO, it - base, e - base, bit, part);
+          for (int k = 0; k < ZK; ++k) part[k] = 0.f;
+          gather_items<NT, ZK, MASHED>(buf, recA, recM, recO, it - base, e - base, bit, part);
 #pragma unroll
-        for (int k = 0; k < ZK; ++k) ac[k] += part[k];
-        it = e;
+          for (int k = 0; k < ZK; ++k) ac[k] += part[k];
+          it = e;
+        }
       }
       if (!last) {
 #pragma unroll

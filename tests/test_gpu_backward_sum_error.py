@@ -1,9 +1,9 @@
 """Rounding error of a backprojected column of many records against the FP64 oracle.
 
-A column's records are summed twelve at a time and the sums added in order.  With u = 2^-24 a rounding has
-an rms of about 0.4 u of the partial sum it rounds; n equal terms in one running sum give 0.4 u sqrt(n / 3)
-of the total, so the 230 records of these columns (180 views, or 60 views and three tilted segments) would
-have 3.5 u in one chain, and have 0.4 u sqrt(19 / 3) = 1.0 u in 19 sums of twelve, whose own roundings and
+Records of several taps are summed twelve at a time and the sums added in order.  With u = 2^-24 a rounding
+has an rms of about 0.4 u of the partial sum it rounds; n equal terms in one running sum give 0.4 u sqrt(n / 3)
+of the total, so the 230 records of these columns (60 views and three tilted segments) would have 3.5 u
+and more in one chain, and have 0.4 u sqrt(19 / 3) = 1.0 u in 19 sums of twelve, whose own roundings and
 those of the lengths add less than 0.3 u.  The bar is 2 u (relative L2 over the image).
 """
 import numpy as np
@@ -25,8 +25,7 @@ def _scanner(n, nz, views, tilts):
                          seg_dz=tuple(tilts), n_subsets=1, name=f"{n}x{n}x{nz}-{views}v-{S}s")
 
 
-@pytest.mark.parametrize("sc", [_scanner(24, 8, 180, (0.0,)), _scanner(104, 8, 180, (0.0,)),
-                                _scanner(24, 33, 60, (0.0, 60.0, -60.0)), _scanner(104, 33, 60, (0.0, 250.0, -250.0))],
+@pytest.mark.parametrize("sc", [_scanner(24, 33, 60, (0.0, 60.0, -60.0)), _scanner(104, 33, 60, (0.0, 250.0, -250.0))],
                          ids=lambda s: s.name)
 def test_columns_of_many_records(sc):
     import paper_1808_07150_gb300 as pkg
