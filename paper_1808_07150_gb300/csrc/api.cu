@@ -677,6 +677,7 @@ int spdhg_create(const spdhg_geometry* geom, spdhg_ctx** out) {
   d.nx = g.nx;
   d.ny = g.ny;
   d.nz = g.nz;
+  d.R = R;
   d.V = V;
   d.m = g.n_subsets;
   d.bins = g.subset_kind == SPDHG_SUBSETS_BINS ? 1 : 0;
@@ -713,7 +714,6 @@ int spdhg_create(const spdhg_geometry* geom, spdhg_ctx** out) {
   if ((e = cudaMemcpy(ctx->d_view_inv, view_inv.data(), sizeof(float2) * V, cudaMemcpyHostToDevice)) != cudaSuccess) return cleanup_fail(e);
   if ((e = cudaMemcpy(ctx->d_tasks, tasks.data(), sizeof(int4) * tasks.size(), cudaMemcpyHostToDevice)) != cudaSuccess) return cleanup_fail(e);
 
-  d.R = R;
   d.P = P;
   d.mashed = mashed ? 1 : 0;
   d.comp = ctx->d_comp;

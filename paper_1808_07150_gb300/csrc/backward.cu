@@ -13,11 +13,15 @@ namespace spdhg {
 void backward_layout(DevGeom& g, const SegDev* seg, CompDev* comp, std::vector<int2>& slots, std::vector<BwdBatch>& batches) {
   const double inv = g.inv_drp;
   const int pad = g.taps - 1;
+  // The ends of a footprint are FP32: with d the image's diagonal, |s| <= d / 2 pixels comes with at most five
+  // roundings of it and four of half its size (products, directions, sum, half width, 1 / d_radial), the bin with one
+  // of R / 2; a margin below that would drop bins that cut a corner (8192 pixels at nine bins a pixel: 0.0113).
+  g.bw_margin = fmaxf(kBinMargin, (float)(ldexp(1.0, -24) * (4.0 * sqrt((double)g.nx * g.nx + (double)g.ny * g.ny) * inv + g.R)));
   auto rows = [&](int cpw) {
     // a tile of 2 cpw x 4 pixels projects onto 2 cpw |c| + 4 |s| pixels of s, at most the tile's
     // diagonal; the kernel widens the row range by twice its bin margin on both sides
     const double diag = sqrt(4.0 * cpw * cpw + 16.0);
-    return (int)floor(diag * inv * (1.0 + 1e-5) + 4.0 * kBinMargin) + 1;
+    return (int)floor(diag * inv * (1.0 + 1e-5) + 4.0 * g.bw_margin) + 1;
   };
   // Runs of staged planes.  A component whose bins hold every plane of its range has its own run,
   // followed by a frame of taps - 1 zeros.  One that holds every second plane is staged without the
@@ -56,7 +60,7 @@ void backward_layout(DevGeom& g, const SegDev* seg, CompDev* comp, std::vector<i
   const long long tiles4 = (long long)((g.nx + 7) / 8) * ((g.ny + 3) / 4);
   g.bw_cpw = tiles4 >= 2 * 152 && (size_t)rows(4) * widest * sizeof(float) <= 80 * 1024 ? 4 : 1;
   g.bw_rows = rows(g.bw_cpw);
-  g.bw_cand = (int)floor(1.41422 * inv + 2.0 * kBinMargin) + 1;
+  g.bw_cand = (int)floor(1.41422 * inv + 2.0 * g.bw_margin) + 1;
   // batches of components whose staged rows fit the buffer: 36 KB leave room for four blocks per SM
   // (171 x 171 x 92, three segments: 36 KB 97.7 us, 44 KB 108.7, 24 KB 115)
   const int room = 36 * 1024 / (int)sizeof(float) / g.bw_rows;

@@ -13,7 +13,7 @@ constexpr int kBwdFill = 32;      // item records a warp holds at a time (one pe
 constexpr size_t kPairBytes = 48 * 1024;   // most of the warps' pair lists: what a kernel has without opting in
 constexpr size_t kBwdMaxSmem = 220 * 1024;
 constexpr int kSumItems = 12;     // records of several taps a column sums before the sum joins the others
-constexpr float kBinMargin = 0.01f;   // radial bins: covers the FP32 rounding of the footprint ends
+constexpr float kBinMargin = 0.01f;   // radial bins: least margin of the footprint ends (backward_layout)
 
 // A (bin, pixel interval) pair: the LOR lines of radial bin r of one view of the stage that cross
 // a voxel column; row is the bin's row among the staged rows.
@@ -29,8 +29,8 @@ __device__ __forceinline__ int tile_rows(const DevGeom& g, const float4 cs, int 
   const float Ym = (float)ty0 + 0.5f * (float)TY - 0.5f * (float)g.ny;
   const float mid = Xm * cs.x + Ym * cs.z;
   const float hw = 0.5f * ((float)TX * fabsf(cs.x) + (float)TY * fabsf(cs.z));
-  *r_min = max(0, (int)ceilf((mid - hw) * g.inv_drp + g.half_R - 2.f * kBinMargin));
-  return min(g.R - 1, min(*r_min + g.bw_rows - 1, (int)floorf((mid + hw) * g.inv_drp + g.half_R + 2.f * kBinMargin)));
+  *r_min = max(0, (int)ceilf((mid - hw) * g.inv_drp + g.half_R - 2.f * g.bw_margin));
+  return min(g.R - 1, min(*r_min + g.bw_rows - 1, (int)floorf((mid + hw) * g.inv_drp + g.half_R + 2.f * g.bw_margin)));
 }
 
 // The stages of a subset: its views are cut into groups of near-equal size.
@@ -61,8 +61,8 @@ __device__ __forceinline__ int warp_pairs(const DevGeom& g, int subset, int l0, 
       const float hw = 0.5f * (fabsf(cs.x) + fabsf(cs.z));
       const float Xc = (float)ix + 0.5f - 0.5f * (float)g.nx;
       const float sc = Xc * cs.x + Yc * cs.z;
-      const int r = (int)ceilf((sc - hw) * g.inv_drp + g.half_R - kBinMargin) + cand;
-      const int rhi = (int)floorf((sc + hw) * g.inv_drp + g.half_R + kBinMargin);
+      const int r = (int)ceilf((sc - hw) * g.inv_drp + g.half_R - g.bw_margin) + cand;
+      const int rhi = (int)floorf((sc + hw) * g.inv_drp + g.half_R + g.bw_margin);
       if (r >= r_min && r <= r_max && r <= rhi) {
         ok = pixel_interval(g, make_line(g, v, r), ix, iy, P.I);
         P.r = r;

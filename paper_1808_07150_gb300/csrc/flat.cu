@@ -113,8 +113,8 @@ __global__ void __launch_bounds__(256) k_backward_flat(const __grid_constant__ D
       const int v = subset_view(g, subset, l);
       const float4 cs = g.view[v];
       const float hw = 0.5f * (fabsf(cs.x) + fabsf(cs.z)), sc = Xc * cs.x + Yc * cs.z;
-      const int r1 = min(g.R - 1, (int)floorf((sc + hw) * g.inv_drp + g.half_R + kBinMargin));
-      for (int r = max(0, (int)ceilf((sc - hw) * g.inv_drp + g.half_R - kBinMargin)); r <= r1; ++r) {
+      const int r1 = min(g.R - 1, (int)floorf((sc + hw) * g.inv_drp + g.half_R + g.bw_margin));
+      for (int r = max(0, (int)ceilf((sc - hw) * g.inv_drp + g.half_R - g.bw_margin)); r <= r1; ++r) {
         PixInt I;
         float len[4];
         if (pixel_interval(g, make_line(g, v, r), ix, iy, I) && segment_taps<1>(g, r, 0, I, len) == 0)

@@ -65,6 +65,7 @@ struct DevGeom {
   // copies (slot, plane) and zero slots
   int bw_cpw, bw_rows, bw_cand, bw_nb, bw_views, bw_buf;
   int bw_step2;          // 1: some component has step 2
+  float bw_margin;       // radial bins by which the FP32 ends of a footprint are widened
   const BwdBatch* bw_batch;
   const int2* bw_slots;
   int n_tasks;           // plane tasks of the forward projector, segment-major

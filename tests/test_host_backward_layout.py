@@ -21,11 +21,11 @@ from paper_1808_07150_gb300 import _build_ext
 HELPER = r"""
 #include "backward.cuh"
 using namespace spdhg;
-// in: nx ny nz V m bins taps; seg_n[n_seg]; comps (seg, qlo, qhi, smask); out: cpw rows cand views batches, most
-// bytes of the pair lists and of a launch
+// in: nx ny nz V m bins taps R; seg_n[n_seg]; comps (seg, qlo, qhi, smask); out: cpw rows cand views batches, most
+// bytes of the pair lists and of a launch, margin in 2^-40 bins
 extern "C" void layout(const int* in, float inv, int n_seg, const int* seg_n, int n_comp, const int* comps, long long* out) {
   DevGeom g{};
-  g.nx = in[0], g.ny = in[1], g.nz = in[2], g.V = in[3], g.m = in[4], g.bins = in[5], g.taps = in[6];
+  g.nx = in[0], g.ny = in[1], g.nz = in[2], g.V = in[3], g.m = in[4], g.bins = in[5], g.taps = in[6], g.R = in[7];
   g.inv_drp = inv, g.n_seg = n_seg, g.n_comp = n_comp;
   std::vector<SegDev> seg(n_seg);
   std::vector<CompDev> comp(n_comp);
@@ -40,6 +40,7 @@ extern "C" void layout(const int* in, float inv, int n_seg, const int* seg_n, in
   out[5] = (long long)bwd_pair_bytes(g);
   out[6] = (long long)bwd_smem(g, g.taps, zk, false, false, g.bw_step2);
   out[7] = kBwdMaxSmem;
+  out[8] = llrint(ldexp((double)g.bw_margin, 40));
 }
 extern "C" unsigned word(int row_slot, int* jp, int* len, int taps, int lanes, int pad, int step2) {
   return item_word(row_slot, *jp, *len, taps, lanes, pad, step2 != 0);
@@ -64,12 +65,12 @@ def helper(tmp_path_factory):
 def layout(helper):
     fn = helper.layout
 
-    def run(nx, ny, nz, inv, views, subsets, taps, seg_n, comps, bins=0):
+    def run(nx, ny, nz, inv, views, subsets, taps, seg_n, comps, bins=0, radial=0):
         a = lambda v: np.ascontiguousarray(v, np.int32).ctypes.data_as(ctypes.POINTER(ctypes.c_int))
         head, sn, cm, out = [np.ascontiguousarray(v, np.int32) for v in
-                             ([nx, ny, nz, views, subsets, bins, taps], seg_n, comps)] + [np.zeros(8, np.int64)]
+                             ([nx, ny, nz, views, subsets, bins, taps, radial or int(1.5 * max(nx, ny) * inv) + 3], seg_n, comps)] + [np.zeros(9, np.int64)]
         fn(a(head), ctypes.c_float(inv), len(sn), a(sn), len(cm), a(cm), out.ctypes.data_as(ctypes.POINTER(ctypes.c_longlong)))
-        return dict(zip(("cpw", "rows", "cand", "views", "batches", "pairs", "smem", "limit"), out.tolist()))
+        return dict(zip(("cpw", "rows", "cand", "views", "batches", "pairs", "smem", "limit", "margin"), out.tolist()))
 
     return run
 
@@ -98,9 +99,10 @@ def test_every_admitted_geometry_fits_its_launches(layout):
 @pytest.mark.parametrize("inv", [0.4, 1.0, 3.0, 9.1])
 @pytest.mark.parametrize("n", [(344, 344), (171, 130), (23, 37)])
 def test_staged_rows_and_candidates_cover_every_footprint(layout, n, inv):
-    f, margin = np.float32, np.float32(0.01)
+    f = np.float32
     nx, ny = n
     L = layout(nx, ny, 4, inv, 24, 2, 1, [4], [(0, 0, 4, 0)])
+    margin = f(math.ldexp(L["margin"], -40))
     assert L["cpw"] == (4 if nx > 100 else 1)
     TX, TY = 2 * L["cpw"], 4
     R = int(1.5 * max(n) * inv) + 3
@@ -156,3 +158,23 @@ def test_record_words_name_their_kind_and_slots(helper, lanes, step2):
                             assert (slot == row_slot + ((at + add) // 2 if step2 else at))[want].all()
                         more = (w & 3) if not step2 else (w >> 1) & 1
                         assert more == ((taps - 1 if not step2 else taps > 2) if seen else 0)
+
+
+@pytest.mark.parametrize("inv", [1.0, 9.1])
+@pytest.mark.parametrize("n", [344, 3413, 8192, 18900])
+def test_margin_covers_the_rounding_of_footprint_ends(layout, n, inv):
+    f = np.float32
+    R = int(1.42 * n * inv) + 3
+    L = layout(n, n, 1, inv, 180, 2, 1, [1], [(0, 0, 1, 0)], radial=R)
+    margin = math.ldexp(L["margin"], -40)
+    assert margin < 0.1 and (n > 344 or margin == f(0.01))
+    rng = np.random.default_rng(n)
+    v, ix, iy = rng.integers(0, 180, 300000), rng.integers(0, n, 300000), rng.integers(0, n, 300000)
+    c, s = np.cos(np.pi * v / 180), np.sin(np.pi * v / 180)
+    cf, sf = c.astype(f), s.astype(f)
+    hw = f(0.5) * (np.abs(cf) + np.abs(sf))
+    sc = (ix.astype(f) + f(0.5) - f(0.5 * n)) * cf + (iy.astype(f) + f(0.5) - f(0.5 * n)) * sf
+    mid, half = ((ix + 0.5 - 0.5 * n) * c + (iy + 0.5 - 0.5 * n) * s) * inv + 0.5 * (R - 1), 0.5 * (np.abs(c) + np.abs(s)) * inv
+    for sign in (-1, 1):
+        end = (sc + f(sign) * hw) * f(inv) + f(0.5 * (R - 1))
+        assert np.abs(end.astype(np.float64) - (mid + sign * half)).max() < margin
