@@ -286,7 +286,8 @@ enum { SPDHG_TUNE_PRIOR_COLS = 0,   /* prior kernel: voxel columns per block, in
                                        (blocks of up to 32 warps) */
        SPDHG_TUNE_PRIOR_YCHUNK = 1, /* prior kernel: rows marched per block */
        SPDHG_TUNE_FWD_SPLIT = 2,    /* forward kernel: row parts of one LOR line (partial sums
-                                       reduced in a fixed order) */
+                                       reduced in a fixed order).  This and the other forward knobs
+                                       have no effect where images and lines have one slice and plane */
        SPDHG_TUNE_FWD_WARPS = 3,    /* forward kernel: plane tasks per block (1, 2, 4, 8 or 16, at
                                        most 12 are used); a warp owns one task of up to four words
                                        of 32 planes of one segment, so a line's tasks are spread
@@ -303,8 +304,9 @@ enum { SPDHG_TUNE_PRIOR_COLS = 0,   /* prior kernel: voxel columns per block, in
                                        taking every k-th pixel entry of the line (1 .. 8; their
                                        partial sums are added in a fixed order); 0 = enough for
                                        four warps per block when a line has few plane tasks */
-       SPDHG_TUNE_PRIOR_VZ = 7,     /* accepted (1, 2 or 4) without effect: a thread of the prior
-                                       kernel holds one voxel */
+       SPDHG_TUNE_PRIOR_VZ = 7,     /* accepted (1, 2 or 4); a thread of the prior kernel holds one voxel,
+                                       and the value only enters the check of SPDHG_TUNE_PRIOR_COLS:
+                                       cols * ceil(nz / (32 vz)) may not exceed 32 */
        SPDHG_TUNE_KNOBS = 8 };
 
 /* Sets one launch-shape knob of the context (value 0: default).  Out-of-range values are rejected

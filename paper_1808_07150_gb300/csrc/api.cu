@@ -668,7 +668,9 @@ int spdhg_create(const spdhg_geometry* geom, spdhg_ctx** out) {
     comp[c].jhi = -(int)floor(f - span) + 2;
     fz_lo = std::max(fz_lo, comp[c].jhi + taps - 1);
   }
-  // plane q (read as min(q, n - 1)) reads slabs q - j0 - t: the highest is n - 1 - jlo
+  // plane q reads slabs q - j0 - t: the highest is n - 1 - jlo.  The lanes of a word past the segment's last plane
+  // read up to 31 floats further, into the next column or the 32 floats the launch adds after the
+  // last one; their sums are not written.
   for (int c = 0; c < C; ++c) fz_stride = std::max(fz_stride, g.seg_n[c_seg[c]] + 3 - comp[c].jlo);
   fz_lo = (fz_lo + 3) & ~3;  // 16-byte copies of aligned columns
   fz_stride += fz_lo;

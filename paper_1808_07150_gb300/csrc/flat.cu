@@ -33,7 +33,9 @@ bool flat_geometry(const DevGeom& g) { return g.nz == 1 && g.P == 1 && g.n_comp 
 
 // Forward: `per_line` warps share a line, a lane takes every 32 per_line-th row of the dominant axis; the
 // lanes' sums are added by a fixed tree, the warps' in order.  Bound: latency of one chain (table loads,
-// a row's intervals, x, the bin's data).  64 x 64, 9 views x 95 bins: 14.9 -> 6.5 us.
+// a row's intervals, x, the bin's data).  64 x 64, 9 views x 95 bins: 14.9 -> 6.5 us.  One warp up to 32 rows, two up to
+// 64 (64 x 64, 9 views x 96 bins: 10.1, 8.3, 9.9 us with 1, 2, 4), then four: 128 x 128 14.0, 12.2, 13.3 us, 256 x 256 24.5,
+// 24.7, 25.4 us with 1, 2, 4, level within a tenth, and the shortest chain where an image is far longer.
 template <int MODE>
 __global__ void __launch_bounds__(128) k_forward_flat(const __grid_constant__ DevGeom g, int subset, int lines, int per_line,
                                                       const __grid_constant__ FwdArgs a) {

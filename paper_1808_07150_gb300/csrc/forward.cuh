@@ -166,7 +166,8 @@ __device__ __forceinline__ void forward_epilogue(const DevGeom& g, const FwdArgs
 // compacted); the entries are then processed in chunks: the x columns of chunk c+1 are copied to
 // shared memory (cp.async, 16 bytes at a time where the columns are aligned) inside zero frames wide
 // enough for every tap of every plane of the segments (the axial bound of the geometry, so no plane
-// needs a range test), and its axial taps computed while chunk c is accumulated.  One tap record
+// needs a range test; lanes past a segment's last plane read up to 31 floats beyond their frame, hence the
+// 32 spare floats after the last column, and are not written), and its axial taps computed while chunk c is accumulated.  One tap record
 // serves all words of a task, packed FP32 FMAs accumulate two words.  Mashed geometries sum the
 // components of the segment one after the other, each kept by the planes that include it, and a chunk's
 // component sums before they join the bin's (each joining by itself, a bin of nine components came to 2.7
@@ -190,7 +191,7 @@ __global__ void __launch_bounds__(kFwdMaxWarps * 32, GROUPS ? 3 : 2)
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int scan_scratch[33];
   const int FL = g.fz_lo, xs_stride = g.fz_stride;
-  float* xs = reinterpret_cast<float*>(smem);                                        // [2][chunk][xs_stride] + 32
+  float* xs = reinterpret_cast<float*>(smem);                                        // [2][chunk][xs_stride] + 32 spare
   float2* recA = reinterpret_cast<float2*>(xs + 2 * chunk * xs_stride + 32);         // [2][ncomp_tab][chunk]
   MoreLengths<NT>* recB = reinterpret_cast<MoreLengths<NT>*>(recA + 2 * ncomp_tab * chunk);
   Entry* ent = reinterpret_cast<Entry*>(recB + (NT > 1 ? 2 * ncomp_tab * chunk : 0));  // [ecap]

@@ -198,7 +198,7 @@ struct PriorArgs {
 };
 cudaError_t launch_prior(const DevGeom& g, const PriorArgs& a, cudaStream_t s);
 // whether the prior kernel's launch-shape knobs fit together
-bool prior_launch_ok(const DevGeom& g, int kind);
+bool prior_launch_ok(const DevGeom& g);
 
 struct TgvArgs {
   int block;             // 0: A = (grad, -I), 1: A = (0, E)

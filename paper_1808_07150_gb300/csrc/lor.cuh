@@ -136,19 +136,6 @@ __device__ __forceinline__ int segment_taps(const DevGeom& g, int r, int ci, con
   return j0l - in0;
 }
 
-// Asynchronous global -> shared copies (4 and 16 bytes).
-__device__ __forceinline__ void cp_async4(float* dst, const float* src) {
-  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(d), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async16(float* dst, const float* src) {
-  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit_wait_all() {
-  asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;\n" ::: "memory");
-}
-
 // Block-wide exclusive prefix sum of one int per thread (blockDim <= 1024); returns the
 // exclusive prefix and writes the total to *total.  Uses `scratch` (>= 33 ints of shared).
 __device__ __forceinline__ int block_exclusive_scan(int v, int* scratch, int* total) {

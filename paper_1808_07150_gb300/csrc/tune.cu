@@ -152,11 +152,11 @@ extern "C" int spdhg_autotune(spdhg_ctx* ctx, int reps, int* chosen, void* strea
     int best = keep;
     // the current setting is the one to beat (a candidate list need not hold the built-in choice)
     double best_ms = INFINITY;
-    if (k.forward || prior_launch_ok(ctx->dg, ctx->params.prior))
+    if (k.forward || prior_launch_ok(ctx->dg))
       if (int st = time_kernel(ctx, k.forward, reps, s, tm, &best_ms)) return st;
     for (int v : k.values) {
       if (spdhg_tune(ctx, k.id, v) != SPDHG_OK) continue;
-      if (!k.forward && !prior_launch_ok(ctx->dg, ctx->params.prior)) continue;
+      if (!k.forward && !prior_launch_ok(ctx->dg)) continue;
       double ms = 0.0;
       if (int st = time_kernel(ctx, k.forward, reps, s, tm, &ms)) {
         spdhg_tune(ctx, k.id, keep);

@@ -10,9 +10,10 @@
 // Storage: BF16 channels-last activations (element (v, c) at p[v * stride + off + c]); the
 // encoder output of level l < L-1 is written straight into the right half of the decoder's
 // concatenation buffer, the transposed convolution into its left half.  Every convolution
-// (forward, data gradient, weight gradient) runs on the tensor cores (igemm.cu); weights are
-// FP32 masters with BF16 copies in the layouts the GEMM operands need (forward [co][tap][ci],
-// flipped for the data gradient [ci][tap][co]).  Weight gradients are reduced deterministically
+// (forward, data gradient, weight gradient) runs on the tensor cores (igemm.cu, conv3.cuh); weights are
+// FP32 masters with BF16 copies in the layouts the operands need: 3x3x3 tap by tap in core matrices, forward and
+// flipped for the data gradient (256 input channels: forward [co][tap][ci]); 2x2x2 [child][co][ci] and
+// [ci][child][co].  Weight gradients are reduced deterministically
 // (partial sums per reduction split, then a fixed-order sum).
 #include <cuda_bf16.h>
 #include <math.h>
