@@ -215,10 +215,10 @@ __device__ __forceinline__ float ld_now(const float* p) {
 // warps overlaps the gathers of the others.  Between stages the sums rest in shared memory; with one
 // stage in all (SINGLE) they never leave registers.
 //
-// Bound: instruction issue (77 % active at the mMR scale; the gather is half of the 80 M warp
+// Bound: instruction issue (76 % active at the mMR scale; the gather is half of the 82 M warp
 // instructions, the rest is set-up, staging, records and the epilogue), so four columns share a
 // warp's set-up and several views share a stage.  Measured on GB300: 344 x 344 x 127 voxels, one
-// view of 344 x 837 bins, BWD_UPDATE 137 -> 99 us (302 MB algorithmic, 3.1 TB/s) against a block of
+// view of 344 x 837 bins, BWD_UPDATE 137 -> 100 us (302 MB algorithmic, 3.0 TB/s) against a block of
 // 16 one-column warps whose epilogues ran in step; 171 x 171 x 92, 12-13 views x 250 planes,
 // 128 -> 95 us; 128 x 128 x 64, 8-9 views, three mashed components, 51 -> 36 us; 64 x 64 x 1, 9 views,
 // 19 -> 12 us; 344 x 344 x 127, one view, 121 components over 837 planes (BWD_OUT) 767 -> 747 us
