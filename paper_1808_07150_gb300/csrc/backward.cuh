@@ -10,7 +10,7 @@ namespace spdhg {
 
 constexpr int kBwdWarps = 8;      // warps per block: 2 in x, 4 in y, CPW columns in x each
 constexpr int kBwdFill = 32;      // item records a warp holds at a time (one per lane)
-constexpr size_t kPairBytes = 48 * 1024;   // most of the warps' pair lists: what a kernel has without opting in
+constexpr size_t kPairBytes = 48 * 1024;   // most of the warps' pair lists: what a kernel has by default
 constexpr size_t kBwdMaxSmem = 220 * 1024;
 constexpr int kSumItems = 12;     // records of several taps a column sums before the sum joins the others
 constexpr float kBinMargin = 0.01f;   // radial bins: least margin of the footprint ends (backward_layout)
@@ -620,6 +620,8 @@ cudaError_t backward_items_nt(const DevGeom& g, int pass, unsigned short* cnt, u
   const dim3 t = bwd_tiles(g), grid(t.x, t.y, g.m * groups);
   const size_t smem = bwd_pair_bytes(g);
   auto go = [&](auto kern) {
+    cudaError_t e = allow_dynamic_smem(kern, smem);
+    if (e != cudaSuccess) return e;
     kern<<<grid, kBwdWarps * 32, smem, s>>>(g, groups, cnt, bad, starts, stage_base, items, hdr);
     return cudaGetLastError();
   };

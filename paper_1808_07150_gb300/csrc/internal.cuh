@@ -76,7 +76,7 @@ struct DevGeom {
   int tune[SPDHG_TUNE_KNOBS];  // launch-shape overrides (0: built-in heuristic)
 };
 
-// Lets `kern` take more than 48 KB of dynamic shared memory.  The attribute belongs to the
+// Lets `kern` take more than 48 KB of shared memory with `smem` bytes of it dynamic.  The attribute belongs to the
 // function, not to a launch, so it is raised once per device to the largest value the function
 // admits (the opt-in maximum less its static shared memory) instead of to this launch's size:
 // launches and captured graph nodes of contexts with different sizes then never invalidate one
@@ -84,7 +84,7 @@ struct DevGeom {
 cudaError_t allow_dynamic_smem_fn(const void* kern, size_t smem);
 template <class K>
 cudaError_t allow_dynamic_smem(K kern, size_t smem) {
-  if (smem <= 48 * 1024) return cudaSuccess;
+  if (smem <= 47 * 1024) return cudaSuccess;  // the 48 KB hold static shared memory too (below 1 KB in every kernel)
   return allow_dynamic_smem_fn(reinterpret_cast<const void*>(kern), smem);
 }
 

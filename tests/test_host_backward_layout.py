@@ -1,8 +1,8 @@
 """Launch layout of the backprojector, checked on the CPU with the library's own host code.
 
 * backward_layout chooses tile, views per stage and staged rows; for every geometry spdhg_create admits
-  (vx / d_radial up to 9.1, up to 256 slices) the pair lists stay within the 48 KB a kernel has without
-  opting in and the whole launch within the limit of k_backward.
+  (vx / d_radial up to 9.1, up to 256 slices) the pair lists stay within the 48 KB a kernel has by
+  default and the whole launch within the limit of k_backward.
 * Its staged rows and candidate bins cover every bin whose lines cross a pixel of the tile, by
   brute force over the kernel's FP32 formulas and the exact footprints.
 * An item's record word names its kind and the staged slots of its lanes for components whose planes lie
